@@ -8,6 +8,7 @@
 #include "fft.cuh"
 #include "fft2.cuh"
 #include "erode_plan.h"
+#include "erode_stream.h"
 #include "fft_plan.h"
 #include "orient_order.h"
 #include "sweep_bits.cuh"
@@ -149,4 +150,24 @@ extern "C" void imf_host_orient_order(const double *R, int n, int spread, int *o
     std::vector<int> o = imf::locality_order(r, n);
     if (spread) o = imf::spread_order(o);
     for (int i = 0; i < n; ++i) out[i] = o[i];
+}
+
+// The plan of the streamed minimum over sharp points (erode_stream.h) of one orientation's sharp
+// offsets. head gets P, R, Q, stages, tile x, rows, W, plane groups, axis, lists, rows and 16-byte
+// columns copied, ox, ou, ow; words the descriptor words. Returns the number of words, -1 where the
+// plan refuses the points and -2 when the output array is too small.
+extern "C" int imf_host_plan_stream(const int *sh, int n_pts, const int *K, int *head, int max_words,
+                                    int *words_out)
+{
+    std::vector<std::vector<int32_t>> v(1, std::vector<int32_t>(sh, sh + 3 * (size_t)n_pts));
+    std::vector<imf::EsOrient> h;
+    std::vector<int> words;
+    imf::EsGeometry g;
+    if (!imf::es_plan(v, K, g, h, words)) return -1;
+    const int out[15] = {g.P, g.R, g.Q, g.stages, imf::kEsTX, imf::kEsRows, imf::kEsW, imf::kEsNW,
+                         h[0].axis, h[0].lists, h[0].rows, h[0].quads, h[0].ox, h[0].ou, h[0].ow};
+    std::memcpy(head, out, sizeof out);
+    if ((int)words.size() > max_words || h[0].words != (int)words.size() || g.words != h[0].words) return -2;
+    std::memcpy(words_out, words.data(), words.size() * sizeof(int));
+    return (int)words.size();
 }

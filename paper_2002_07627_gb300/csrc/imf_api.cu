@@ -27,6 +27,7 @@
 #include "fft2.cuh"
 #include "imf_internal.cuh"
 #include "erode_plan.h"
+#include "erode_stream.h"
 #include "fft_plan.h"
 #include "orient_order.h"
 
@@ -86,6 +87,11 @@ struct Tool {
     size_t erode_smem = 0;
     int erode_bps = 1;                   // resident erosion blocks per SM
     bool erode_levels = false;           // plan and kernel of the dyadic-level minimum (erode3)
+    bool es_ok = false;                  // planned for the streamed minimum (erode_stream.cu)
+    std::vector<signed char> es_axis;    // its run axis of every orientation
+    EsGeometry es;
+    EsOrient *es_head = nullptr;
+    int *es_words = nullptr;
     long n_rt = 0, n_rk = 0, n_sh = 0;
     std::vector<int> perm, iperm;        // internal orientation order -> caller's index, and back
     int *perm_dev = nullptr;             // perm on the device (per-orientation outputs)
@@ -416,6 +422,8 @@ void free_tool(imf_handle h, Tool &t)
     dfree(h, t.er_chunks);
     dfree(h, t.er_chunk_start);
     dfree(h, t.er_runs);
+    dfree(h, t.es_head);
+    dfree(h, t.es_words);
     dfree(h, t.d_taps);
     dfree(h, t.d_bmat);
     dfree(h, t.perm_dev);
@@ -1125,6 +1133,12 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
         return fail(h, IMF_ERR_INVALID_ARG, "sharp-point set too wide for the tiled minimum (%zu bytes of tile)",
                     t.erode_smem);
     }
+    std::vector<EsOrient> es_head;
+    std::vector<int> es_words;
+    t.es_ok = es_plan(t.sh, t.kmax, t.es, es_head, es_words);
+    if (!t.es_ok) { es_head.clear(); es_words.clear(); }
+    t.es_axis.clear();
+    for (const EsOrient &e : es_head) t.es_axis.push_back((signed char)e.axis);
     if (!plan_only) {
         int dev = 0, n = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -1141,7 +1155,8 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
                     vbytes((size_t)t.P[2], 8) + vbytes(rto.size(), 4) + vbytes(rts.size(), 4) +
                     vbytes(ivv.size(), sizeof(int4)) + vbytes(ivst.size(), 4) +
                     vbytes(chunks.size(), sizeof(ErodeChunk)) + vbytes(chst.size(), 4) +
-                    vbytes(eruns.size(), sizeof(int2)) + vbytes(t.perm.size(), 4);
+                    vbytes(eruns.size(), sizeof(int2)) + vbytes(t.perm.size(), 4) +
+                    vbytes(es_head.size(), sizeof(EsOrient)) + vbytes(es_words.size(), 4);
     if (!plan_only) {
         twiddles(t.M, t.M, t.M, tw);
         if ((st = upload(h, &t.twM, tw))) return bail(st);
@@ -1154,7 +1169,8 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
         if ((st = upload(h, &t.rt_off, rto)) || (st = upload(h, &t.rt_start, rts)) ||
             (st = upload(h, &t.sw_pairs, ivv)) || (st = upload(h, &t.sw_start, ivst)) ||
             (st = upload(h, &t.er_chunks, chunks)) || (st = upload(h, &t.er_chunk_start, chst)) ||
-            (st = upload(h, &t.er_runs, eruns)) || (st = upload(h, &t.perm_dev, t.perm)))
+            (st = upload(h, &t.er_runs, eruns)) || (st = upload(h, &t.perm_dev, t.perm)) ||
+            (st = upload(h, &t.es_head, es_head)) || (st = upload(h, &t.es_words, es_words)))
             return bail(st);
     }
     // --- direct tensor-core path: groups, union taps, B matrices
@@ -1261,7 +1277,34 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         if (h->opt.sweep_loop && !h->aset) launch_sweep_loop(a, h->nsm, s);
         else launch_sweep(a, s);
     }
-    {
+    // The streamed kernel from about twelve (tile, orientation) pairs an SM on: below that its blocks are
+    // mostly ring fill. Measured with the tiled one (us, tiles x orientations): 48^3 98 against 87 (1152),
+    // 60x40x90 175 against 174 (1760), 40^3 199 against 215 (1920), 72^3 166 against 197 (2592), 80^3 438
+    // against 582 (11520). Grids of one plane use an eighth of its tiles and stay with the tiled kernel.
+    bool streamed = false;
+    const long es_t = es_tiles(op.nx, op.ny, op.nz);
+    if (t.es_ok && op.erode_xt == 0 && !t.erode_levels && op.nz > 1 && es_t * nb >= 12L * h->nsm) {
+        EsArgs a{};
+        a.g = h->g; a.g_so = gso; a.gpx = t.gpx; a.wx = t.win[0]; a.wy = t.win[1]; a.wz = t.win[2];
+        a.head = t.es_head; a.words = t.es_words;
+        a.nx = op.nx; a.ny = op.ny; a.nz = op.nz; a.orient_base = o0; a.nb = nb;
+        a.f = h->f; a.status = h->dev_small; a.geo = t.es;
+        for (int i = o0; i < o0 + nb; ++i)
+            if (t.es_axis[i] >= 0) a.kind[t.es_axis[i]]++;
+        const long tiles = es_t;
+        // blocks per tile: about six waves of them (a block loads its outputs and fills its ring before
+        // it reduces anything, so fewer and longer blocks win where the tiles alone fill the SMs), and
+        // not below one and a half orientations each. Measured, ms: 256^3 x 64 a launch, 5632 tiles: 17.1
+        // with one block a tile, 17.4 with two, 18.3 with four; 128^3 x 64, 768 tiles: 2.62, 2.48, 2.48;
+        // 48^3 x 24, 48 tiles: 0.105 with four, 0.089 with eight, 0.103 with twelve
+        const long G = op.erode_groups > 0 ? op.erode_groups
+                                           : std::min((6L * h->nsm + tiles - 1) / tiles,
+                                                      (2L * std::max(a.kind[0], a.kind[1]) + 2) / 3);
+        a.ngroups = (int)std::max(1L, std::min(G, (long)nb));
+        Launch L(h, KID_ERODE, s);
+        streamed = launch_erode_stream(a, s);
+    }
+    if (!streamed) {
         Erode2Args a{};
         a.g = h->g; a.g_so = gso; a.gpx = t.gpx; a.gpy = t.win[1];
         a.wx = t.win[0]; a.wy = t.win[1]; a.wz = t.win[2];
