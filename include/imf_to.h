@@ -58,8 +58,10 @@ imf_status imf_to2d_project(imf_to2d h, const float *xi, float *rho, void *cuda_
 /* FEA of the design rho (DEVICE float [nely][nelx]) under the DEVICE FP64 load `force`
  * [2 (nelx+1)(nely+1)] with the DEVICE uint8 dof mask `fixed` (nonzero = clamped, u = 0).
  * Keeps u in the handle (for imf_to2d_sensitivity) and copies it to `u_out` (DEVICE FP64, or
- * NULL). Synchronous: the host checks the residual every few iterations. Compliance, iteration
- * count and relative residual via imf_to2d_result. Errors: IMF_ERR_INVALID_ARG,
+ * NULL). Synchronous. A conjugate gradient preconditioned by one multigrid V-cycle, in one launch;
+ * where that does not reach cg_tol within 600 iterations (or its hierarchy, about 530 bytes a node, found
+ * no memory), a Jacobi-preconditioned one from the start. Compliance, iteration count of the one that
+ * finished and relative residual via imf_to2d_result. Errors: IMF_ERR_INVALID_ARG,
  * IMF_ERR_CUDA; IMF_ERR_TIMEOUT when cg_max_iter is reached before cg_tol (u is the last
  * iterate). */
 imf_status imf_to2d_analyze(imf_to2d h, const float *rho, const double *force, const uint8_t *fixed, double *u_out,
@@ -75,7 +77,7 @@ imf_status imf_to2d_sensitivity(imf_to2d h, const float *xi, const float *rho, f
  * volfrac; passive elements (DEVICE uint8, or NULL) keep xi = 1. S: DEVICE float, >= 0.
  * change_out (HOST, or NULL) receives the mean |xi_new - xi| over the non-passive elements
  * (Alg. 2's volume difference), vol_out (HOST, or NULL) the mean projected density reached.
- * Synchronous (bisection on the host, one volume reduction per step).
+ * Synchronous (one launch; eta above 4 takes a bisection on the host, one volume reduction per step).
  * Errors: IMF_ERR_INVALID_ARG (NULL, volfrac outside (0, 1), move <= 0), IMF_ERR_CUDA. */
 imf_status imf_to2d_update(imf_to2d h, const float *xi, const float *S, const uint8_t *passive, double volfrac,
                            double move, double eta, float *xi_new, double *change_out, double *vol_out,

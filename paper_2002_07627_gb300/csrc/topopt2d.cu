@@ -2,6 +2,11 @@
 // Heaviside projection, matrix-free FEA with a Jacobi-preconditioned conjugate gradient (FP64),
 // compliance sensitivity with its filter, and the optimality-criteria update.
 //
+// The FEA and the update run as cooperative kernels (topopt2d_mg.cu). What stands here beside the entry
+// points takes over where those do not apply: the Jacobi-preconditioned iteration for designs on which the
+// multigrid-preconditioned one does not converge (or whose hierarchy does not fit), and the host's bisection
+// for exponents whose powers would leave the FP64 range.
+//
 // The stiffness operator is applied node by node: a node gathers the contributions of its (up
 // to four) elements, E_e times the rows of the element matrix k0 that belong to its corner, so
 // no atomics are needed. The conjugate gradient keeps its scalars on the device (rotating slots,
@@ -16,11 +21,15 @@
 #include <vector>
 
 #include "imf_to.h"
+#include "topopt2d_mg.cuh"
 
 namespace {
 
 constexpr int kT = 256;
 constexpr int kCheckEvery = 16;      // CG iterations between residual checks on the host
+// multigrid-preconditioned iterations before the plain iteration takes over: designs of the loop take 40 to
+// 150 (256 x 128, contrast 1e3), and these cost what about 800 plain ones do
+constexpr int kMgMaxIter = 600;
 
 // scalar slots: rz[3], pq[2], rr[3], ff, vol, cnt, change
 enum { S_RZ = 0, S_PQ = 3, S_RR = 5, S_FF = 8, S_VOL = 9, S_CNT = 10, S_CHG = 11, S_N = 16 };
@@ -322,6 +331,10 @@ struct imf_to2d_s {
     long ne = 0, ndof = 0;
     double *k0 = nullptr, *E = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr,
            *diag = nullptr, *sc = nullptr, *s = nullptr;
+    void *mem = nullptr;                 // what the pointers above and `bar` lie in
+    void *mg_mem = nullptr;              // multigrid hierarchy, or NULL where it does not fit
+    imf_to::MgArgs mg{};
+    unsigned *bar = nullptr;
     double compliance = 0.0, rel_res = 0.0;
     int iters = 0;
     bool have_u = false;
@@ -381,17 +394,49 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
     h->ndof = 2L * (o->nelx + 1) * (o->nely + 1);
     double k[64];
     element_matrix(o->nu, k);
-    bool ok = cudaMalloc(&h->k0, 64 * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&h->E, h->ne * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&h->s, h->ne * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&h->sc, S_N * sizeof(double)) == cudaSuccess;
-    for (double **v : {&h->x, &h->r, &h->z, &h->p, &h->q, &h->diag})
-        ok = ok && cudaMalloc(v, h->ndof * sizeof(double)) == cudaSuccess;
-    ok = ok && cudaMemcpy(h->k0, k, sizeof k, cudaMemcpyHostToDevice) == cudaSuccess;
-    if (!ok) {
+    // one allocation holds every array (each from a 256-byte boundary)
+    struct Part {
+        void **p;
+        size_t bytes;
+    };
+    const size_t v = h->ndof * sizeof(double), e = h->ne * sizeof(double);
+    const Part parts[] = {{(void **)&h->k0, 64 * sizeof(double)}, {(void **)&h->E, e}, {(void **)&h->s, e},
+                          {(void **)&h->sc, S_N * sizeof(double)}, {(void **)&h->bar, 2 * sizeof(unsigned)},
+                          {(void **)&h->x, v}, {(void **)&h->r, v}, {(void **)&h->z, v}, {(void **)&h->p, v},
+                          {(void **)&h->q, v}, {(void **)&h->diag, v}};
+    size_t total = 0;
+    for (const Part &q : parts) total += (q.bytes + 255) / 256 * 256;
+    if (cudaMalloc(&h->mem, total) != cudaSuccess) {
         cudaGetLastError();
         imf_to2d_destroy(h);
         return IMF_ERR_OOM;
+    }
+    char *at = static_cast<char *>(h->mem);
+    for (const Part &q : parts) {
+        *q.p = at;
+        at += (q.bytes + 255) / 256 * 256;
+    }
+    if (cudaMemcpy(h->k0, k, sizeof k, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaGetLastError();
+        imf_to2d_destroy(h);
+        return IMF_ERR_OOM;
+    }
+    // the hierarchy takes about 530 bytes a node; without it the plain iteration does the work
+    const size_t mg_bytes = imf_to::mg_plan(o->nelx, o->nely, o->nu, h->mg);
+    if (mg_bytes && cudaMalloc(&h->mg_mem, mg_bytes) == cudaSuccess) {
+        imf_to::mg_place(h->mg, h->mg_mem);
+        h->mg.k0 = h->k0;
+        h->mg.E = h->E;
+        h->mg.x = h->x;
+        h->mg.r0 = h->r;
+        h->mg.p0 = h->p;
+        h->mg.p1 = h->z;
+        h->mg.q = h->q;
+        h->mg.sc = h->sc;
+        h->mg.bar = h->bar;
+    } else {
+        h->mg_mem = nullptr;
+        cudaGetLastError();
     }
     *out = h;
     return IMF_OK;
@@ -400,7 +445,8 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
 void imf_to2d_destroy(imf_to2d h)
 {
     if (!h) return;
-    for (double *v : {h->k0, h->E, h->x, h->r, h->z, h->p, h->q, h->diag, h->sc, h->s}) cudaFree(v);
+    cudaFree(h->mem);
+    cudaFree(h->mg_mem);
     delete h;
 }
 
@@ -423,6 +469,29 @@ imf_status imf_to2d_analyze(imf_to2d h, const float *rho, const double *force, c
     const Grid g{o.nelx, o.nely};
     const long nn = (long)(o.nelx + 1) * (o.nely + 1);
     moduli_kernel<<<blocks(h->ne), kT, 0, s>>>(rho, h->E, h->ne, o.E0, o.Emin, o.penal);
+    if (h->mg_mem) {
+        imf_to::MgArgs a = h->mg;
+        a.force = force;
+        a.fixed = fixed;
+        a.tol2 = o.cg_tol * o.cg_tol;
+        a.max_iter = o.cg_max_iter < kMgMaxIter ? o.cg_max_iter : kMgMaxIter;
+        TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
+        TO_CU(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), s));
+        imf_to::mg_setup(a, s);
+        TO_CU(imf_to::mg_solve(a, s));
+        if (u_out) TO_CU(cudaMemcpyAsync(u_out, h->x, h->ndof * sizeof(double), cudaMemcpyDeviceToDevice, s));
+        double res[imf_to::kScN];
+        TO_CU(cudaMemcpyAsync(res, h->sc, sizeof res, cudaMemcpyDeviceToHost, s));
+        TO_CU(cudaStreamSynchronize(s));
+        if (res[imf_to::kScDone] == 1.0) {
+            h->compliance = res[imf_to::kScC];
+            h->iters = (int)res[imf_to::kScIt];
+            h->rel_res = res[imf_to::kScFf] > 0 ? std::sqrt(res[imf_to::kScLast] / res[imf_to::kScFf]) : 0.0;
+            h->have_u = true;
+            return IMF_OK;
+        }
+    }
+    // plain iteration, from the start
     diag_kernel<<<blocks(nn), kT, 0, s>>>(g, h->k0, h->E, fixed, h->diag);
     TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
     cg_init_kernel<<<blocks(h->ndof), kT, 0, s>>>(h->ndof, force, fixed, h->diag, h->x, h->r, h->z, h->p, h->sc);
@@ -486,6 +555,28 @@ imf_status imf_to2d_update(imf_to2d h, const float *xi, const float *S, const ui
         return fail(h, IMF_ERR_INVALID_ARG, "volfrac %g / move %g / eta %g out of range", volfrac, move, eta);
     cudaStream_t s = (cudaStream_t)stream;
     const double beta = h->opt.beta;
+    if (eta <= 4.0) {
+        // one launch: the multiplier's bracket [1e-12, 1e12] is bisected on the device, where only the powers
+        // lam^-eta matter; within eta = 4 they and S^eta stay inside the FP64 range for any float S
+        imf_to::OcArgs a{};
+        a.n = h->ne; a.xi = xi; a.S = S; a.passive = passive; a.volfrac = volfrac; a.move = move; a.eta = eta; a.beta = beta;
+        a.li_lo = std::pow(1e-12, -eta);
+        a.li_hi = std::pow(1e12, -eta);
+        for (double ratio = 1e24; ratio > 1.0 + 1e-9; ratio = std::sqrt(ratio)) ++a.steps;
+        a.xs = h->s; a.out = xi_new; a.sc = h->sc; a.bar = h->bar;
+        TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
+        TO_CU(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), s));
+        TO_CU(imf_to::oc_solve(a, s));
+        double r[6];
+        unsigned bar[2];
+        TO_CU(cudaMemcpyAsync(r, h->sc, sizeof r, cudaMemcpyDeviceToHost, s));
+        TO_CU(cudaMemcpyAsync(bar, h->bar, sizeof bar, cudaMemcpyDeviceToHost, s));
+        TO_CU(cudaStreamSynchronize(s));
+        if (bar[1]) return fail(h, IMF_ERR_TIMEOUT, "optimality-criteria update: a grid barrier timed out");
+        if (change_out) *change_out = r[3] > 0 ? r[4] / r[3] : 0.0;
+        if (vol_out) *vol_out = r[3] > 0 ? r[5] / r[3] : 0.0;
+        return IMF_OK;
+    }
     double res[3] = {0, 0, 0};
     auto volume = [&](double lam, float *out) -> imf_status {
         TO_CU(cudaMemsetAsync(h->sc + S_VOL, 0, 3 * sizeof(double), s));

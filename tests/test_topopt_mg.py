@@ -1,0 +1,103 @@
+"""The cooperative kernels of the 2D optimisation loop: the multigrid-preconditioned conjugate
+gradient against the oracle's direct solve, and the update's bisection against the oracle's, at the
+sizes where the hierarchy changes shape."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _need():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2002_07627_gb300 import binding, build
+    build.build()
+    return binding
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# one element; the coarsest grid alone; one level inside a block; thin strips; odd and even extents on
+# both sides of the block-wide and grid-wide levels; clamped dofs anywhere
+@pytest.mark.parametrize("nx,ny", [(1, 1), (3, 7), (4, 4), (9, 1), (1, 40), (31, 31), (32, 31), (37, 23), (130, 3),
+                                   (64, 64), (101, 67), (256, 128)])
+@pytest.mark.parametrize("clamp", ["edge", "scattered"])
+def test_multigrid_cg_matches_the_direct_solve(nx, ny, clamp):
+    """The residual of the returned displacements is the iteration's 1e-11 |f| plus what its recurrence
+    can drift from the true one in FP64, at most about eps |K| |u| an iteration (Greenbaum's bound; on the
+    long strips |u| reaches 1e9 |f|, and the direct solve's own residual is 1e-8 |f|); displacements and
+    compliance agree with the direct solve."""
+    binding = _need()
+    from oracle import to2d
+    rng = np.random.default_rng(nx * 1000 + ny)
+    rho = rng.uniform(0.0, 1.0, (ny, nx)).astype(np.float32)
+    ndof = 2 * (nx + 1) * (ny + 1)
+    fixed = np.zeros(ndof, np.uint8)
+    if clamp == "edge":
+        left = np.arange(ny + 1) * (nx + 1)
+        fixed[2 * left] = fixed[2 * left + 1] = 1
+    else:
+        fixed[rng.choice(ndof, max(3, ndof // 9), replace=False)] = 1
+        fixed[[0, 1]] = 1                    # no rigid motion left
+        fixed[ndof - 1] = 1
+    force = rng.standard_normal(ndof)
+    to = binding.To2d(nx, ny, cg_tol=1e-11)
+    # a force at an odd FP64 offset: the caller's arrays carry no alignment beyond their type
+    buf = torch.empty(ndof + 1, dtype=torch.float64, device="cuda")
+    f_d = buf[1:]
+    f_d.copy_(_dev(force))
+    u_d = torch.empty(ndof, dtype=torch.float64, device="cuda")
+    c, it, res = to.analyze(_dev(rho), f_d, _dev(fixed), u_d)
+    u_o, c_o, K = to2d.fea(rho.astype(np.float64), force, fixed.astype(bool))
+    free = fixed == 0
+    u = u_d.cpu().numpy()
+    assert res <= 1e-11 and it > 0
+    r = (K @ u - force)[free]
+    drift = it * np.finfo(np.float64).eps * abs(K).sum(0).max() * np.linalg.norm(u)
+    assert np.linalg.norm(r) <= 1.1e-11 * np.linalg.norm(force[free]) + drift
+    scale = max(np.abs(u_o).max(), 1e-300)
+    assert np.abs(u - u_o).max() <= 1e-6 * scale and np.all(u[~free] == 0)
+    assert abs(c - c_o) <= 1e-7 * max(abs(c_o), 1e-300)
+    to.close()
+
+
+def test_iteration_cap_is_reported_with_the_last_iterate():
+    binding = _need()
+    from paper_2002_07627_gb300 import synth
+    force, fixed, _ = synth.cantilever2d(48, 24)
+    rho = torch.full((24, 48), 0.5, device="cuda")
+    to = binding.To2d(48, 24, cg_max_iter=2)
+    u = torch.zeros(force.shape, dtype=torch.float64, device="cuda")
+    with pytest.raises(binding.ImfError) as e:
+        to.analyze(rho, _dev(force), _dev(fixed), u)
+    assert e.value.status == 4 and float(u.abs().max()) > 0
+    to.close()
+
+
+@pytest.mark.parametrize("nx,ny,eta", [(1, 1, 0.5), (7, 3, 0.5), (64, 40, 0.3), (256, 128, 0.5), (40, 20, 5.0)])
+@pytest.mark.parametrize("passive", [False, True])
+def test_update_on_the_device_matches_the_oracle(nx, ny, eta, passive):
+    """xi_new to FP32 storage (1e-6 also covers the last step of the bisection, 1e-9 in the multiplier);
+    eta = 5 takes the host's bisection."""
+    binding = _need()
+    from oracle import to2d
+    rng = np.random.default_rng(nx + 7 * ny)
+    xi = rng.uniform(0.0, 1.0, (ny, nx)).astype(np.float32)
+    S = np.exp(rng.standard_normal((ny, nx))).astype(np.float32)
+    S[rng.uniform(size=S.shape) < 0.1] = 0.0
+    pas = None
+    if passive and nx > 1:
+        pas = np.zeros((ny, nx), np.uint8)
+        pas[:, 0] = 1
+        xi[:, 0] = 1.0
+    to = binding.To2d(nx, ny)
+    out = torch.empty((ny, nx), device="cuda")
+    change, vol = to.update(_dev(xi), _dev(S), None if pas is None else _dev(pas), 0.5, out, move=0.2, eta=eta)
+    x_o, _, vol_o = to2d.oc_update(xi, S, 0.5, 2.0, pas, 0.2, eta)
+    free = np.ones(xi.shape, bool) if pas is None else pas == 0
+    assert np.abs(out.cpu().numpy() - x_o).max() <= 1e-6
+    assert abs(vol - vol_o) <= 1e-7 and abs(change - np.abs(x_o - xi)[free].mean()) <= 1e-6
+    to.close()
