@@ -240,7 +240,7 @@ imf_status imf_compute_accessible_sets(imf_handle h, const float *rho_omega, con
  *   order, removed : HOST int / int64 [max_steps]: set index and voxels removed per step.
  *   n_steps    : HOST out, steps taken; negative / left (or NULL): HOST out, |N| and the
  *                voxels no set can reach (inaccessible negative space).
- * Synchronous (one count per step is read back). Uses handle-owned scratch (grown on demand).
+ * Synchronous (one launch). Uses handle-owned scratch (grown on demand).
  * Errors: IMF_ERR_INVALID_ARG (NULL, n_sets < 1, max_steps < 0), IMF_ERR_OOM, IMF_ERR_CUDA. */
 imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, const float *rho_omega,
                             const uint8_t *fixture, int max_steps, int *order, long long *removed, int *n_steps,

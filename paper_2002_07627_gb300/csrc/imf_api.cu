@@ -1573,11 +1573,13 @@ imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, cons
         TRY(dalloc(h, &h->plan_rem, (size_t)words));
         h->plan_rem_n = (size_t)words;
     }
-    if ((size_t)n_sets + 1 > h->plan_cnt_n) {
+    // counters (three sets in turn), barrier, results, removed voxels and order, in 8-byte words
+    const size_t nc = 3 * ((size_t)n_sets + 1), need = nc + 1 + 3 + (size_t)n_sets + ((size_t)n_sets + 1) / 2;
+    if (need > h->plan_cnt_n) {
         dfree(h, h->plan_cnt);
         h->plan_cnt_n = 0;
-        TRY(dalloc(h, &h->plan_cnt, (size_t)n_sets + 1));
-        h->plan_cnt_n = (size_t)n_sets + 1;
+        TRY(dalloc(h, &h->plan_cnt, need));
+        h->plan_cnt_n = need;
     }
     h->last_stream = s;
     h->used_stream = true;
@@ -1585,45 +1587,31 @@ imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, cons
         Launch L(h, KID_PLAN, s);
         launch_plan_init(rho_omega, fixture, op.nx, op.ny, op.nz, (int)awords, op.tau, h->plan_rem, s);
     }
-    std::vector<unsigned long long> cnt(n_sets);
-    auto counts = [&]() -> imf_status {
-        CU(cudaMemsetAsync(h->plan_cnt, 0, sizeof(unsigned long long) * n_sets, s));
-        {
-            Launch L(h, KID_PLAN, s);
-            launch_plan_count(sets, words, n_sets, h->plan_rem, h->plan_cnt, s);
-        }
-        CU(cudaMemcpyAsync(cnt.data(), h->plan_cnt, sizeof(unsigned long long) * n_sets, cudaMemcpyDeviceToHost, s));
-        CU(cudaStreamSynchronize(s));
-        return IMF_OK;
-    };
-    // size of the negative space: popcount(remaining & remaining), in the counter after the sets'
-    unsigned long long total = 0;
-    CU(cudaMemsetAsync(h->plan_cnt + n_sets, 0, sizeof total, s));
+    PlanArgs a{};
+    a.sets = sets; a.words = words; a.n_sets = n_sets; a.max_steps = max_steps; a.rem = h->plan_rem;
+    a.counts = h->plan_cnt;
+    a.bar = reinterpret_cast<unsigned *>(h->plan_cnt + nc);
+    a.result = reinterpret_cast<long long *>(h->plan_cnt + nc + 1);
+    a.removed = a.result + 3;
+    a.order = reinterpret_cast<int *>(a.removed + n_sets);
+    CU(cudaMemsetAsync(h->plan_cnt, 0, (nc + 1) * sizeof(unsigned long long), s));
     {
         Launch L(h, KID_PLAN, s);
-        launch_plan_count(h->plan_rem, words, 1, h->plan_rem, h->plan_cnt + n_sets, s);
+        CU(launch_plan_greedy(a, s));
     }
-    CU(cudaMemcpyAsync(&total, h->plan_cnt + n_sets, sizeof total, cudaMemcpyDeviceToHost, s));
+    // barrier words, results, removed voxels and order come back in one copy
+    std::vector<long long> out(need - nc);
+    CU(cudaMemcpyAsync(out.data(), h->plan_cnt + nc, out.size() * sizeof(long long), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
-    unsigned long long rest = total;
-    int k = 0;
-    while (k < max_steps && rest > 0) {
-        TRY(counts());
-        int best = 0;
-        for (int i = 1; i < n_sets; ++i)
-            if (cnt[i] > cnt[best]) best = i;
-        if (cnt[best] == 0) break;
-        order[k] = best;
-        removed[k] = (long long)cnt[best];
-        rest -= cnt[best];
-        ++k;
-        Launch L(h, KID_PLAN, s);
-        launch_plan_remove(sets + (long)best * words, words, h->plan_rem, s);
-    }
-    CU(cudaStreamSynchronize(s));
+    unsigned bar[2];
+    std::memcpy(bar, out.data(), sizeof bar);
+    if (bar[1]) return fail(h, IMF_ERR_TIMEOUT, "process plan: a grid barrier timed out");
+    const int k = (int)out[1];
     *n_steps = k;
-    if (negative) *negative = (long long)total;
-    if (left) *left = (long long)rest;
+    std::memcpy(removed, out.data() + 4, k * sizeof(long long));
+    std::memcpy(order, out.data() + 4 + n_sets, k * sizeof(int));
+    if (negative) *negative = out[2];
+    if (left) *left = out[3];
     return IMF_OK;
 }
 

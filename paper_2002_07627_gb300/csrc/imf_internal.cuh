@@ -177,11 +177,19 @@ void launch_sweep_loop(const SweepArgs &a, int nsm, cudaStream_t s);
 // remaining[w] = bits of the negative space Omega_0 and [rho <= tau] in word w of [nz][ny][awords]
 void launch_plan_init(const float *rho, const uint8_t *fix, int nx, int ny, int nz, int awords, double tau,
                       uint32_t *remaining, cudaStream_t s);
-// counts[s] += popcount(sets[s] & remaining) for s < n_sets (counts zeroed by the caller)
-void launch_plan_count(const uint32_t *sets, long set_words, int n_sets, const uint32_t *remaining,
-                       unsigned long long *counts, cudaStream_t s);
-// remaining &= ~sets[pick]
-void launch_plan_remove(const uint32_t *set, long words, uint32_t *remaining, cudaStream_t s);
+// The greedy plan on those words, one cooperative launch.
+struct PlanArgs {
+    const uint32_t *sets;        // [n_sets][words]
+    long words;
+    int n_sets, max_steps;
+    uint32_t *rem;               // remaining negative space, cleared as the plan goes
+    unsigned long long *counts;  // 3 (n_sets + 1), zeroed by the caller
+    unsigned *bar;               // grid barrier, two words, zeroed by the caller
+    int *order;                  // min(max_steps, n_sets)
+    long long *removed;          // as long as order
+    long long *result;           // steps, |N|, what is left
+};
+cudaError_t launch_plan_greedy(const PlanArgs &a, cudaStream_t s);
 
 
 // Tiled minimum over sharp points: erode.cuh.

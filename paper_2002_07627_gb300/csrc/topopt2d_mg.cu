@@ -23,11 +23,14 @@
 #include <algorithm>
 #include <cmath>
 
+#include "grid_barrier.cuh"
 #include "topopt2d_mg.cuh"
 
 namespace imf_to {
 
 namespace {
+
+using imf::GridBarrier;
 
 constexpr int T = kMgThreads;
 constexpr int kHalo = 464;               // nodes of a staged tile with its halo
@@ -58,47 +61,6 @@ template <typename F> __device__ __forceinline__ double scalar(F &&f, double *sl
     __syncthreads();
     return v;
 }
-
-__device__ __forceinline__ unsigned long long now_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Barrier over the grid (cooperative launch): false once it, or another block's, gave up.
-struct GridBarrier {
-    unsigned *bar;
-    unsigned target = 0;
-    __device__ __forceinline__ bool wait()
-    {
-        __shared__ unsigned bad;
-        target += gridDim.x;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(bar, 1u);
-            unsigned v, b = 0;
-            unsigned long long t0 = 0;
-            for (unsigned n = 0;; ++n) {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-                if ((int)(v - target) >= 0) break;
-                if ((n & 255u) == 255u) {
-                    if (!t0) t0 = now_ns();
-                    if (now_ns() - t0 > 5000000000ull || *(volatile unsigned *)(bar + 1)) {
-                        b = 1;
-                        atomicExch(bar + 1, 1u);
-                        break;
-                    }
-                }
-            }
-            __threadfence();
-            bad = b;
-        }
-        __syncthreads();
-        return bad == 0;
-    }
-};
 
 // ------------------------------------------------------------------------------------- set-up
 // stencil of the finest level from the element matrix and the moduli
@@ -738,19 +700,6 @@ __global__ void __launch_bounds__(T) oc_solve_kernel(const __grid_constant__ OcA
     }
 }
 
-template <typename A> cudaError_t launch_cooperative(void (*kernel)(A), const A &args, long work, cudaStream_t s)
-{
-    int dev = 0, sms = 0, per = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, T, 0);
-    if (e != cudaSuccess) return e;
-    const long most = (long)std::max(per, 1) * sms, want = (work + T - 1) / T;
-    void *p[1] = {const_cast<A *>(&args)};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kernel), dim3((unsigned)std::max(1L, std::min(most, want))),
-                                       dim3(T), p, 0, s);
-}
-
 int blocks(long n) { return (int)std::max(1L, std::min((n + 127) / 128, 65535L)); }
 
 } // namespace
@@ -830,8 +779,8 @@ void mg_setup(const MgArgs &a, cudaStream_t s)
 cudaError_t mg_solve(const MgArgs &a, cudaStream_t s)
 {
     const MgLevel &l = a.lv[0];
-    return launch_cooperative(mg_solve_kernel, a, (long)((l.nx + l.tw) / l.tw) * ((l.ny + l.th) / l.th) * T, s);
+    return imf::launch_cooperative(mg_solve_kernel, a, T, (long)((l.nx + l.tw) / l.tw) * ((l.ny + l.th) / l.th), s);
 }
-cudaError_t oc_solve(const OcArgs &a, cudaStream_t s) { return launch_cooperative(oc_solve_kernel, a, a.n, s); }
+cudaError_t oc_solve(const OcArgs &a, cudaStream_t s) { return imf::launch_cooperative(oc_solve_kernel, a, T, (a.n + T - 1) / T, s); }
 
 } // namespace imf_to

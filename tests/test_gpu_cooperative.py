@@ -1,6 +1,6 @@
-"""The cooperative kernels of the 2D optimisation loop: the multigrid-preconditioned conjugate
-gradient against the oracle's direct solve, and the update's bisection against the oracle's, at the
-sizes where the hierarchy changes shape."""
+"""The cooperative kernels: the multigrid-preconditioned conjugate gradient and the update of the 2D
+optimisation loop against the oracle's, at the sizes where the hierarchy changes shape, and the greedy
+process plan."""
 import numpy as np
 import pytest
 
@@ -101,3 +101,27 @@ def test_update_on_the_device_matches_the_oracle(nx, ny, eta, passive):
     assert np.abs(out.cpu().numpy() - x_o).max() <= 1e-6
     assert abs(vol - vol_o) <= 1e-7 and abs(change - np.abs(x_o - xi)[free].mean()) <= 1e-6
     to.close()
+
+
+@pytest.mark.parametrize("shape,n_sets,max_steps", [((1, 1, 1), 1, None), ((3, 5, 33), 7, None), ((9, 40, 97), 70, None),
+                                                    ((9, 40, 97), 70, 3), ((2, 2, 31), 2100, None), ((40, 60, 70), 5, 0)])
+def test_greedy_plan_matches_the_oracle_on_given_sets(shape, n_sets, max_steps):
+    """Steps, counts and rest on random sets (some empty, some equal, so that ties occur), with and
+    without a cap, and with more sets than one pass counts: whole numbers, so equal."""
+    binding = _need()
+    import oracle
+    rng = np.random.default_rng(n_sets)
+    nz, ny, nx = shape
+    sets = rng.uniform(size=(n_sets,) + shape) < rng.choice([0.0, 0.02, 0.3], n_sets)[:, None, None, None]
+    sets[n_sets // 2] = sets[0]
+    words = -(-nx // 32)
+    padded = np.zeros((n_sets, nz, ny, words * 32), bool)
+    padded[..., :nx] = sets
+    packed = np.packbits(padded, axis=-1, bitorder="little").view(np.int32)
+    rho = rng.uniform(0, 1, shape).astype(np.float32)
+    fix = (rng.uniform(size=shape) < 0.1).astype(np.uint8)
+    imf = binding.Imf(shape)
+    steps, neg, left = imf.process_plan(_dev(packed), _dev(rho), _dev(fix), max_steps)
+    want = oracle.process_plan(list(sets), (fix == 0) & (rho <= 0.5), max_steps)
+    assert (steps, neg, left) == want
+    imf.close()
