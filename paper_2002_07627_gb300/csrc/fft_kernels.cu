@@ -250,7 +250,10 @@ void launch_axis_fft(int sign, const AxisArgs &a, int nbatch, int norient, cudaS
 
 void launch_rfft_fwd(const RfftArgs &a, cudaStream_t s)
 {
-    const int lw = x_log_rows(a.M), W = 1 << lw;
+    // fewer rows a block where 32 of them would leave SMs without one (same arithmetic per row)
+    int lw = x_log_rows(a.M);
+    while (lw > 3 && (a.rows >> lw) < 2 * 152) --lw;
+    const int W = 1 << lw;
     const size_t smem = x_smem(a.M, W);
     dim3 grid((a.rows + W - 1) / W);
     if (lw == 5) { set_smem(rfft_fwd_kernel<5>, smem); rfft_fwd_kernel<5><<<grid, kThreads, smem, s>>>(a); }

@@ -145,7 +145,8 @@ struct imf_handle_s {
     int2 *flags = nullptr;
     int flag_cap = 0;
     int *dev_small = nullptr;   // [0] status, [1] flag count of the batch, [2] maxbits,
-                                // [3] maxbits (penalize), [4] flags of the last compute
+                                // [3] maxbits (penalize), [4] flags of the last compute,
+                                // [5] blocks of the penalty done
     // host staging for imf_compute_host
     float *h_rho = nullptr, *h_fbar = nullptr, *h_raw = nullptr;
     uint8_t *h_fix = nullptr, *h_sec = nullptr, *h_acc = nullptr;
@@ -734,6 +735,11 @@ void axis_opts(imf_handle h, AxisArgs &a)
     a.status = h->dev_small;
 }
 
+// One z-plane, unpadded (2D): the z transforms are the identity. The forward y pass then writes the spectrum
+// and the inverse y pass forms the spectral product on its loads; the separate z passes, of a length that no
+// kernel is shaped for, took 64 of 290 us for two tools at 256 x 128.
+bool planar(const Tool &t) { return t.P[2] == 1 && t.win[2] == 1; }
+
 // forward 3D real FFT of a real grid [nz][ny][nx] (optionally min(1, x + fixture)) into the
 // half spectrum [Pz][Py][Hs] of plan `t`, using X1 / X2 as intermediates
 imf_status forward_real_3d(imf_handle h, const Tool &t, const float *src, const uint8_t *fix, int nx, int ny, int nz,
@@ -752,11 +758,15 @@ imf_status forward_real_3d(imf_handle h, const Tool &t, const float *src, const 
         a.in = X1; a.in_sb = (long)ny * t.Hs; a.in_sl = t.Hs;
         a.out = X2; a.out_sb = (long)t.P[1] * t.Hs; a.out_sl = t.Hs;
         a.nx = t.Hx; a.lin = ny; a.j0 = 0; a.lout = t.P[1]; a.scale = 1.f; a.tw = t.twy; a.plan = t.ply;
+        if (planar(t)) {
+            // one plane: the z transform is the identity, so this pass ends in the spectrum
+            a.out = out; a.scale = scale; a.conj_out = conj_out;
+        }
         set_split(h, a, t.sy); axis_opts(h, a);
         Launch L(h, KID_AXIS_FWD, s);
         launch_axis_fft(-1, a, nz, 1, s);
     }
-    {
+    if (!planar(t)) {
         AxisArgs a{};
         a.in = X2; a.in_sb = t.Hs; a.in_sl = (long)t.P[1] * t.Hs;
         a.out = out; a.out_sb = t.Hs; a.out_sl = (long)t.P[1] * t.Hs;
@@ -1344,17 +1354,20 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
     h->used_stream = true;
     int *status = h->dev_small, *fcount = h->dev_small + 1;
     unsigned *maxbits = (unsigned *)(h->dev_small + 2);
-    {
-        Launch L(h, KID_INIT, s);
-        launch_fill_f32(h->f, INFINITY, N, s);
-    }
     // the accessible output: from the minimum when that is exact (one tool, sharp points = the
     // whole cutter), else by the sweep; neither when the caller does not ask for it
     const bool acc_from_f = acc && !op.accessible_by_sweep && h->n_tools == 1 && h->tools[0].sharp_is_cutter;
     h->run_sweep = (acc && !acc_from_f) || h->aset != nullptr;
-    if (h->run_sweep) CU(cudaMemsetAsync(h->A, 0, sizeof(uint32_t) * (size_t)op.nz * op.ny * h->awords, s));
-    CU(cudaMemsetAsync(maxbits, 0, sizeof(unsigned), s));
-    CU(cudaMemsetAsync(h->dev_small + 4, 0, sizeof(int), s));
+    {
+        Launch L(h, KID_INIT, s);
+        launch_init(h->f, N, h->run_sweep ? h->A : nullptr, (long)op.nz * op.ny * h->awords, h->dev_small, s);
+    }
+    bool fresh = true;          // the batch's near-threshold count is still zero from the launch above
+    auto zero_count = [&]() -> imf_status {
+        if (op.recheck && !fresh) CU(cudaMemsetAsync(fcount, 0, sizeof(int), s));
+        fresh = false;
+        return IMF_OK;
+    };
     for (int ti = 0; ti < h->n_tools; ++ti) {
         const Tool &t = h->tools[ti];
         const long gso_ = (long)t.win[2] * t.win[1] * t.gpx;
@@ -1367,7 +1380,7 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
             }
             for (size_t gi = 0; gi + 1 < t.grp_start.size(); ++gi) {
                 const int o0 = t.grp_start[gi], nb = t.grp_start[gi + 1] - o0;
-                if (op.recheck) CU(cudaMemsetAsync(fcount, 0, sizeof(int), s));
+                TRY(zero_count());
                 {
                     DirectArgs a{};
                     a.rhohl = h->rhohl; a.PX = t.dP[0]; a.PY = t.dP[1]; a.PZ = t.dP[2];
@@ -1407,8 +1420,8 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
         const long spso = (long)t.P[2] * t.P[1] * t.Hs;
         for (int o0 = 0; o0 < t.n_orient; o0 += h->slots) {
             const int nb = std::min(h->slots, t.n_orient - o0);
-            if (op.recheck) CU(cudaMemsetAsync(fcount, 0, sizeof(int), s));
-            {
+            TRY(zero_count());
+            if (!planar(t)) {
                 AxisArgs a{};
                 a.in = t.spec + spso * o0; a.in_so = spso; a.in_sb = t.Hs; a.in_sl = (long)t.P[1] * t.Hs;
                 a.mul = h->rho_spec; a.mul_so = 0; a.mul_sb = t.Hs; a.mul_sl = (long)t.P[1] * t.Hs;
@@ -1422,6 +1435,10 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
             ay.in = h->Y1; ay.in_so = y1so; ay.in_sb = (long)t.P[1] * t.Hs; ay.in_sl = t.Hs;
             ay.out = h->Y2; ay.out_so = y2so; ay.out_sb = (long)t.win[1] * t.Hs; ay.out_sl = t.Hs;
             ay.nx = t.Hx; ay.lin = t.P[1]; ay.j0 = 0; ay.lout = t.win[1]; ay.scale = 1.f; ay.tw = t.twy; ay.plan = t.ply;
+            if (planar(t)) {
+                ay.in = t.spec + spso * o0; ay.in_so = spso;
+                ay.mul = h->rho_spec; ay.mul_so = 0; ay.mul_sb = (long)t.P[1] * t.Hs; ay.mul_sl = t.Hs;
+            }
             set_split(h, ay, t.sy); axis_opts(h, ay);
             IrfftArgs ax{};
             ax.in = h->Y2; ax.in_sy = t.Hs; ax.in_sz = (long)t.win[1] * t.Hs; ax.in_so = y2so;
@@ -1434,12 +1451,14 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
             ax.orient_base = o0; ax.M = t.M; ax.twM = t.twM; ax.twP = t.twP; ax.plan = t.plM;
             set_split(h, ax, t.sM);
             ax.write_bits = h->run_sweep || h->keep_g;
-            if (!op.separate_yx_passes && yx2_fits(ay, ax, t.Hs)) {
+            // the fused pass has a block per plane and slot: a planar grid's few planes leave most SMs idle (8
+            // planes of 160 x 142: 30 us), and the two passes, which split planes further, are faster
+            if (!op.separate_yx_passes && !planar(t) && yx2_fits(ay, ax, t.Hs)) {
                 Launch L(h, KID_YX, s);
                 launch_yx2_threshold(ay, ax, t.Hs, t.win[2], nb, s);
             } else {
                 {
-                    Launch L(h, KID_AXIS_INV, s);
+                    Launch L(h, ay.mul ? KID_AXIS_INV_MUL : KID_AXIS_INV, s);
                     launch_axis_fft(1, ay, t.win[2], nb, s);
                 }
                 Launch L(h, KID_IRFFT_THRESH, s);
@@ -1522,14 +1541,14 @@ imf_status imf_penalize_sensitivity(imf_handle h, float *sens, const float *rho_
     unsigned *mb = (unsigned *)(h->dev_small + 3);
     h->last_stream = s;
     h->used_stream = true;
-    CU(cudaMemsetAsync(mb, 0, sizeof(unsigned), s));
+    // the maximum's word is zero between calls: allocated so, and cleared by the kernel that reads it
     {
         Launch L(h, KID_ABSMAX, s);
         launch_absmax_omega0(sens, fixture, N, mb, s);
     }
     {
         Launch L(h, KID_PENALIZE, s);
-        launch_penalize(sens, rho_omega, imf_bar, secluded, N, mb, w_acc, h->opt.tau, s);
+        launch_penalize(sens, rho_omega, imf_bar, secluded, N, mb, (unsigned *)(h->dev_small + 5), w_acc, h->opt.tau, s);
     }
     CU(cudaGetLastError());
     return IMF_OK;

@@ -234,7 +234,8 @@ void launch_rho_hl(const float *rho, const uint8_t *fix, int nx, int ny, int nz,
 bool launch_direct(const DirectArgs &a, int nsm, cudaStream_t s);
 int run_mma_selftest(const uint16_t *A, const uint16_t *B, float *D, int N, int K, int *status, cudaStream_t s);
 
-void launch_fill_f32(float *p, float v, long n, cudaStream_t s);
+// f = infinity, A = 0 (where given), small[1], [2], [4] = 0
+void launch_init(float *f, long n, uint32_t *A, long words, int *small, cudaStream_t s);
 void launch_max_omega0(const float *f, const uint8_t *fix, long n, unsigned *maxbits, cudaStream_t s);
 struct FinalizeArgs {
     const float *f;
@@ -254,7 +255,7 @@ struct FinalizeArgs {
 void launch_finalize(const FinalizeArgs &a, cudaStream_t s);
 void launch_absmax_omega0(const float *v, const uint8_t *fix, long n, unsigned *maxbits, cudaStream_t s);
 void launch_penalize(float *sens, const float *rho, const float *fbar, const uint8_t *sec, long n,
-                     const unsigned *maxbits, double w, double tau, cudaStream_t s);
+                     unsigned *maxbits, unsigned *done, double w, double tau, cudaStream_t s);
 
 // Eq. eq_filtered_sens with the filter of Eq. eq_accFilter at one voxel (FP32):
 // S = (1 - w) S_phi / m + w S_IMF with S_IMF = f_bar where rho > tau, 1 on Gamma, 0 elsewhere;

@@ -381,9 +381,15 @@ __global__ void __launch_bounds__(256) recheck_blocks_kernel(RecheckArgs a)
     }
 }
 
-__global__ void fill_f32_kernel(float *p, float v, long n)
+// Start of a compute, one launch: the running minimum at infinity, the accessible bits (where the sweep
+// builds them) empty, the near-threshold counts and the maximum zero.
+__global__ void init_kernel(float *f, long n, uint32_t *A, long words, int *small)
 {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) p[i] = v;
+    const long first = blockIdx.x * (long)blockDim.x + threadIdx.x, step = (long)gridDim.x * blockDim.x;
+    for (long i = first; i < n; i += step) f[i] = INFINITY;
+    if (A)
+        for (long i = first; i < words; i += step) A[i] = 0u;
+    if (first == 0) small[1] = small[2] = small[4] = 0;
 }
 
 __device__ __forceinline__ float block_max(float v)
@@ -448,13 +454,19 @@ __global__ void finalize_kernel(FinalizeArgs a)
     }
 }
 
-// Eq. eq_filtered_sens with Eq. eq_accFilter (FP32).
+// Eq. eq_filtered_sens with Eq. eq_accFilter (FP32). The block that finishes last clears the maximum for the
+// next call: every block has read it by then.
 __global__ void penalize_kernel(float *sens, const float *rho, const float *fbar, const uint8_t *sec, long n,
-                                const unsigned *maxbits, float w, float tau)
+                                unsigned *maxbits, unsigned *done, float w, float tau)
 {
-    const float m = __uint_as_float(*maxbits);
+    const float m = __uint_as_float(*(volatile unsigned *)maxbits);
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
         sens[i] = penalized_sensitivity(sens[i], rho[i], fbar[i], sec[i], m, w, tau);
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(done, 1u) == gridDim.x - 1) {
+        *maxbits = 0u;
+        *done = 0u;
+    }
 }
 
 } // namespace
@@ -512,9 +524,9 @@ void launch_recheck_blocks(const RecheckArgs &a, int max_points, cudaStream_t s)
     recheck_blocks_kernel<<<blocks, 256, 0, s>>>(a);
 }
 
-void launch_fill_f32(float *p, float v, long n, cudaStream_t s)
+void launch_init(float *f, long n, uint32_t *A, long words, int *small, cudaStream_t s)
 {
-    fill_f32_kernel<<<blocks_for(n), kThreads, 0, s>>>(p, v, n);
+    init_kernel<<<blocks_for(n), kThreads, 0, s>>>(f, n, A, words, small);
 }
 
 void launch_max_omega0(const float *f, const uint8_t *fix, long n, unsigned *maxbits, cudaStream_t s)
@@ -533,9 +545,9 @@ void launch_finalize(const FinalizeArgs &a, cudaStream_t s)
 }
 
 void launch_penalize(float *sens, const float *rho, const float *fbar, const uint8_t *sec, long n,
-                     const unsigned *maxbits, double w, double tau, cudaStream_t s)
+                     unsigned *maxbits, unsigned *done, double w, double tau, cudaStream_t s)
 {
-    penalize_kernel<<<blocks_for(n), kThreads, 0, s>>>(sens, rho, fbar, sec, n, maxbits, (float)w, (float)tau);
+    penalize_kernel<<<blocks_for(n), kThreads, 0, s>>>(sens, rho, fbar, sec, n, maxbits, done, (float)w, (float)tau);
 }
 
 } // namespace imf
