@@ -23,6 +23,9 @@ constexpr int kErThreads = (kErTX / kErXT) * kErTY * kErTZ;
 // threads of a block with xt consecutive x outputs per thread
 __host__ __device__ constexpr int er_threads(int xt) { return (kErTX / xt) * kErTY * kErTZ; }
 constexpr int kErBlocksPerSM = 1024 / kErThreads;            // 64 registers per thread
+// The tiled kernel's block on a grid of one z-plane: 64 x 32 outputs, a lane per row
+constexpr int kErTY2 = 32;
+constexpr int kErThreads2 = kErTX / kErXT * kErTY2;
 // most run descriptors of one chunk (larger chunks are split)
 constexpr int kErMaxRunsPerChunk = 2048;
 // dynamic shared memory of one block (one per SM): a chunk's g tile followed by its run
@@ -49,6 +52,7 @@ struct Erode2Args {
     int orient_base, nb;
     int ngroups;                 // orientation groups per tile (blockIdx.z = group * tiles_z + tile z)
     float *f;
+    bool planar;                 // nz = 1, planned with the planar block
 };
 // xt = consecutive x outputs per thread: 8 (1024 threads, 64 registers each) or 16 (512 threads,
 // 128 registers each); the plan does not depend on it

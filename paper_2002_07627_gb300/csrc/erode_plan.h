@@ -27,13 +27,13 @@ inline bool bank_free(int P, int Q)
 }
 
 // Runs along x (at most maxL long) of the sharp points `sh` (offset triples) of one orientation,
-// grouped in dz-chunks whose g tile and run descriptors fit kErodeBudget bytes together (each
+// of a block of kErTX x ty x tz outputs, grouped in dz-chunks whose g tile and run descriptors fit kErodeBudget bytes together (each
 // chunk takes as many dz as fit, from the largest down); appends the chunks and their (tile
 // offset, length) runs and raises smem_max to the largest tile plus descriptors. K = kmax of the
 // tool's cutter offsets (the translation window starts at t = -K).
 
 inline void plan_erode(const std::vector<int32_t> &sh, const int K[3], std::vector<ErodeChunk> &chunks,
-                std::vector<int2> &runs, size_t &smem_max, int maxL = kErMaxL)
+                std::vector<int2> &runs, size_t &smem_max, int maxL = kErMaxL, int ty = kErTY, int tz = kErTZ)
 {
     if (sh.empty()) return;
     int kmn[3] = {1 << 30, 1 << 30, 1 << 30}, kmx[3] = {-(1 << 30), -(1 << 30), -(1 << 30)};
@@ -57,14 +57,14 @@ inline void plan_erode(const std::vector<int32_t> &sh, const int K[3], std::vect
         }
     }
     const int Ex = kmx[0] - kmn[0] + 1, Ey = kmx[1] - kmn[1] + 1;
-    const int txh = kErTX + Ex - 1, tyh = kErTY + Ey - 1;
+    const int txh = kErTX + Ex - 1, tyh = ty + Ey - 1;
     const int P = txh | 1;
     int Q = tyh * P;
     while (!bank_free(P, Q)) ++Q;
     std::map<int, int> runs_at;                               // dz -> runs
     for (const Run &r : rr) ++runs_at[r.dz];
     const int planes = (int)(kErodeBudget / (4 * (size_t)Q));
-    const int dzc_max = std::max(1, planes - kErTZ + 1);
+    const int dzc_max = std::max(1, planes - tz + 1);
     int dzc = dzc_max;
     for (int hi = kmx[2]; hi >= kmn[2]; hi -= dzc) {
         // the most dz (down from hi) whose tile and descriptors fit the budget together
@@ -75,7 +75,7 @@ inline void plan_erode(const std::vector<int32_t> &sh, const int K[3], std::vect
                 auto it = runs_at.find(z);
                 if (it != runs_at.end()) nr += it->second;
             }
-            const size_t bytes = 4 * (size_t)er_runs_offset(kErTZ + d - 1, Q) +
+            const size_t bytes = 4 * (size_t)er_runs_offset(tz + d - 1, Q) +
                                  8 * (size_t)std::min<long>(nr, kErMaxRunsPerChunk);
             if (bytes > kErodeBudget) break;
             dzc = d;
@@ -101,14 +101,14 @@ inline void plan_erode(const std::vector<int32_t> &sh, const int K[3], std::vect
                 while (ch.run0 + c < ch.run1 && runs[ch.run0 + c].y == L) ++c;
                 ch.lend[L] = c;
             }
-            ch.txh = txh; ch.tyh = tyh; ch.tzh = kErTZ + (hi - lo);
+            ch.txh = txh; ch.tyh = tyh; ch.tzh = tz + (hi - lo);
             ch.pitch_y = P; ch.pitch_z = Q;
             ch.ox = K[0] - kmx[0]; ch.oy = K[1] - kmx[1]; ch.oz = K[2] - hi;
             chunks.push_back(ch);
         }
         for (size_t b = 0; b < cr.size(); b += kErMaxRunsPerChunk) {
             const size_t nr = std::min(cr.size(), b + (size_t)kErMaxRunsPerChunk) - b;
-            smem_max = std::max(smem_max, 4 * (size_t)er_runs_offset(kErTZ + (hi - lo), Q) + 8 * nr);
+            smem_max = std::max(smem_max, 4 * (size_t)er_runs_offset(tz + (hi - lo), Q) + 8 * nr);
         }
     }
 }

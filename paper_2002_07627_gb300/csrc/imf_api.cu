@@ -87,6 +87,7 @@ struct Tool {
     size_t erode_smem = 0;
     int erode_bps = 1;                   // resident erosion blocks per SM
     bool erode_levels = false;           // plan and kernel of the dyadic-level minimum (erode3)
+    bool erode_planar = false;           // planned for the tiled kernel's planar block
     bool es_ok = false;                  // planned for the streamed minimum (erode_stream.cu)
     std::vector<signed char> es_axis;    // its run axis of every orientation
     EsGeometry es;
@@ -1125,12 +1126,15 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
     // the dyadic-level kernel (runs up to kErMaxL3) where every tile row fits its level build,
     // else the pairwise kernel (runs up to kErMaxL)
     t.erode_levels = h->opt.erode_levels != 0;
+    // planar blocks on one z-plane, except for the forms that options select (their plan stays the 3D one)
+    t.erode_planar = h->opt.nz == 1 && h->opt.erode_xt == 0 && !t.erode_levels;
     for (int pass = 0; pass < 2; ++pass) {
         chunks.clear();
         eruns.clear();
         t.erode_smem = 0;
         for (int i = 0; i < n_orient; ++i) {
-            plan_erode(t.sh[i], t.kmax, chunks, eruns, t.erode_smem, t.erode_levels ? kErMaxL3 : kErMaxL);
+            plan_erode(t.sh[i], t.kmax, chunks, eruns, t.erode_smem, t.erode_levels ? kErMaxL3 : kErMaxL,
+                       t.erode_planar ? kErTY2 : kErTY, t.erode_planar ? 1 : kErTZ);
             chst[i + 1] = (int)chunks.size();
         }
         bool rows_fit = true;
@@ -1138,10 +1142,17 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
         if (!t.erode_levels || rows_fit) break;
         t.erode_levels = false;
     }
-    if (t.erode_smem > 227 * 1024) {
+    size_t er_need = t.erode_smem;
+    if (t.erode_planar) {
+        // the widest cutter a tool may have is the 3D block's, whatever block it runs in
+        std::vector<ErodeChunk> c3;
+        std::vector<int2> r3;
+        for (int i = 0; i < n_orient; ++i) plan_erode(t.sh[i], t.kmax, c3, r3, er_need);
+    }
+    if (er_need > 227 * 1024) {
         free_tool(h, t);
         return fail(h, IMF_ERR_INVALID_ARG, "sharp-point set too wide for the tiled minimum (%zu bytes of tile)",
-                    t.erode_smem);
+                    er_need);
     }
     std::vector<EsOrient> es_head;
     std::vector<int> es_words;
@@ -1320,6 +1331,7 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         a.wx = t.win[0]; a.wy = t.win[1]; a.wz = t.win[2];
         a.chunks = t.er_chunks; a.chunk_start = t.er_chunk_start; a.runs = t.er_runs;
         a.nx = op.nx; a.ny = op.ny; a.nz = op.nz; a.orient_base = o0; a.nb = nb; a.f = h->f;
+        a.planar = t.erode_planar;
         // (tile, orientation group) units: at least about twelve waves of resident blocks and
         // at most 16 orientations per block (measured optimum: 8 groups of 8 orientations at
         // 128^3 x 64, 4 groups of 16 at 256^3 with 64 orientations per launch)
@@ -1412,7 +1424,13 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
             }
             continue;
         }
-        TRY(forward_real_3d(h, t, rho, fix, op.nx, op.ny, op.nz, h->X1, h->X2, h->rho_spec, 1.f, 0, s));
+        // the design's spectrum serves every tool of the same padded extents
+        bool have = false;
+        if (ti > 0 && h->tools[ti - 1].path != IMF_BF16_DIRECT) {
+            const Tool &p = h->tools[ti - 1];
+            have = p.P[0] == t.P[0] && p.P[1] == t.P[1] && p.P[2] == t.P[2] && planar(p) == planar(t);
+        }
+        if (!have) TRY(forward_real_3d(h, t, rho, fix, op.nx, op.ny, op.nz, h->X1, h->X2, h->rho_spec, 1.f, 0, s));
         const long y1so = (long)t.win[2] * t.P[1] * t.Hs;
         const long y2so = (long)t.win[2] * t.win[1] * t.Hs;
         const long gso = (long)t.win[2] * t.win[1] * t.gpx;

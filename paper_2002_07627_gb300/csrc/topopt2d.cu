@@ -332,7 +332,7 @@ struct imf_to2d_s {
     double *k0 = nullptr, *E = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr,
            *diag = nullptr, *sc = nullptr, *s = nullptr;
     void *mem = nullptr;                 // what the pointers above and `bar` lie in
-    void *mg_mem = nullptr;              // multigrid hierarchy, or NULL where it does not fit
+    void *mg_mem = nullptr;              // multigrid hierarchy, behind them in `mem`, or NULL where it did not fit
     imf_to::MgArgs mg{};
     unsigned *bar = nullptr;
     double compliance = 0.0, rel_res = 0.0;
@@ -406,7 +406,12 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
                           {(void **)&h->q, v}, {(void **)&h->diag, v}};
     size_t total = 0;
     for (const Part &q : parts) total += (q.bytes + 255) / 256 * 256;
-    if (cudaMalloc(&h->mem, total) != cudaSuccess) {
+    // the multigrid hierarchy (about 530 bytes a node) follows them where it fits; without it the plain
+    // iteration does the work
+    const size_t mg_bytes = imf_to::mg_plan(o->nelx, o->nely, o->nu, h->mg);
+    if (mg_bytes && cudaMalloc(&h->mem, total + mg_bytes) == cudaSuccess) h->mg_mem = static_cast<char *>(h->mem) + total;
+    else cudaGetLastError();
+    if (!h->mg_mem && cudaMalloc(&h->mem, total) != cudaSuccess) {
         cudaGetLastError();
         imf_to2d_destroy(h);
         return IMF_ERR_OOM;
@@ -421,9 +426,7 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
         imf_to2d_destroy(h);
         return IMF_ERR_OOM;
     }
-    // the hierarchy takes about 530 bytes a node; without it the plain iteration does the work
-    const size_t mg_bytes = imf_to::mg_plan(o->nelx, o->nely, o->nu, h->mg);
-    if (mg_bytes && cudaMalloc(&h->mg_mem, mg_bytes) == cudaSuccess) {
+    if (h->mg_mem) {
         imf_to::mg_place(h->mg, h->mg_mem);
         h->mg.k0 = h->k0;
         h->mg.E = h->E;
@@ -434,9 +437,6 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
         h->mg.q = h->q;
         h->mg.sc = h->sc;
         h->mg.bar = h->bar;
-    } else {
-        h->mg_mem = nullptr;
-        cudaGetLastError();
     }
     *out = h;
     return IMF_OK;
@@ -446,7 +446,6 @@ void imf_to2d_destroy(imf_to2d h)
 {
     if (!h) return;
     cudaFree(h->mem);
-    cudaFree(h->mg_mem);
     delete h;
 }
 
@@ -556,25 +555,22 @@ imf_status imf_to2d_update(imf_to2d h, const float *xi, const float *S, const ui
     cudaStream_t s = (cudaStream_t)stream;
     const double beta = h->opt.beta;
     if (eta <= 4.0) {
-        // one launch: the multiplier's bracket [1e-12, 1e12] is bisected on the device, where only the powers
-        // lam^-eta matter; within eta = 4 they and S^eta stay inside the FP64 range for any float S
+        // one launch: only the powers lam^-eta of the multiplier in [1e-12, 1e12] matter there; within eta = 4
+        // they and S^eta stay inside the FP64 range for any float S
         imf_to::OcArgs a{};
         a.n = h->ne; a.xi = xi; a.S = S; a.passive = passive; a.volfrac = volfrac; a.move = move; a.eta = eta; a.beta = beta;
-        a.li_lo = std::pow(1e-12, -eta);
-        a.li_hi = std::pow(1e12, -eta);
-        for (double ratio = 1e24; ratio > 1.0 + 1e-9; ratio = std::sqrt(ratio)) ++a.steps;
         a.xs = h->s; a.out = xi_new; a.sc = h->sc; a.bar = h->bar;
         TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
         TO_CU(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), s));
         TO_CU(imf_to::oc_solve(a, s));
-        double r[6];
+        double r[9];
         unsigned bar[2];
         TO_CU(cudaMemcpyAsync(r, h->sc, sizeof r, cudaMemcpyDeviceToHost, s));
         TO_CU(cudaMemcpyAsync(bar, h->bar, sizeof bar, cudaMemcpyDeviceToHost, s));
         TO_CU(cudaStreamSynchronize(s));
         if (bar[1]) return fail(h, IMF_ERR_TIMEOUT, "optimality-criteria update: a grid barrier timed out");
-        if (change_out) *change_out = r[3] > 0 ? r[4] / r[3] : 0.0;
-        if (vol_out) *vol_out = r[3] > 0 ? r[5] / r[3] : 0.0;
+        if (change_out) *change_out = r[6] > 0 ? r[7] / r[6] : 0.0;
+        if (vol_out) *vol_out = r[6] > 0 ? r[8] / r[6] : 0.0;
         return IMF_OK;
     }
     double res[3] = {0, 0, 0};

@@ -7,8 +7,8 @@
 // two FP64 multiply-adds per SM and clock), with a host round trip every sixteen. On the 256 x 128 cantilever
 // midway in its loop that was 5500 iterations of 24.8 us, 136.8 ms; here 92 of about 50 us, 5.3 ms with the
 // set-up, bound by the grid barriers (eight an iteration) and the latency of the short phases between them.
-// The update's bisection took 36 host round trips, 1.0 ms; in one launch it is 0.17 ms, bound by the FP64
-// exponentials of the projected density.
+// The update's bisection took 36 host round trips, 1.0 ms; in one launch 0.17 ms, and with Newton steps about
+// 0.03 ms, bound by the FP64 exponentials of the projected density and the grid barriers.
 //
 // The iteration itself (operator, vectors, scalar products, stopping rule) is FP64 as before; only the
 // preconditioner, which steers the search directions and not what they converge to, works in FP32: at
@@ -657,46 +657,69 @@ __global__ void __launch_bounds__(T) oc_solve_kernel(const __grid_constant__ OcA
         if (!(a.passive && a.passive[i])) cnt += 1.0;
     }
     cnt = block_sum(cnt, red);
-    if (threadIdx.x == 0) atomicAdd(a.sc + 3, cnt);
+    if (threadIdx.x == 0) atomicAdd(a.sc + 6, cnt);
     if (!g.wait()) return;
-    const double target = a.volfrac * __ldcg(a.sc + 3);
+    const double target = a.volfrac * __ldcg(a.sc + 6);
     // the update at the multiplier whose power lam^-eta is li: xi (S / lam)^eta within the move limit and
-    // [0, 1]; the sum of the projected densities of the free elements, and with `write` also xi_new and
-    // sum |xi_new - xi|
-    auto sum = [&](double li, bool write, double &chg) {
+    // [0, 1]; the sum of the projected densities of the free elements and its slope in log lam, and with
+    // `write` also xi_new and sum |xi_new - xi| (in place of the slope)
+    auto sum = [&](double li, bool write, double &second) {
         double vol = 0.0;
-        chg = 0.0;
+        second = 0.0;
         for (long i = first; i < a.n; i += step) {
             const bool pas = a.passive && a.passive[i];
-            const double x = a.xi[i];
-            double v = a.xs[i] * li;
-            v = fmin(v, fmin(1.0, x + a.move));
+            const double x = a.xi[i], w = a.xs[i] * li;
+            double v = fmin(w, fmin(1.0, x + a.move));
             v = fmax(v, fmax(0.0, x - a.move));
             if (write) a.out[i] = pas ? 1.f : (float)v;
             if (pas) continue;
-            vol += 1.0 - exp(-a.beta * v) + v * eb;
-            if (write) chg += fabs(v - x);
+            const double e = exp(-a.beta * v);
+            vol += 1.0 - e + v * eb;
+            if (write) second += fabs(v - x);
+            else if (v == w) second -= a.eta * v * (a.beta * e + eb);
         }
         return vol;
     };
-    // bisection of the multiplier in log space: the power of sqrt(lo hi) is the root of the powers
-    double lo = a.li_lo, hi = a.li_hi, chg;
-    for (int k = 0; k < a.steps; ++k) {
-        const double mid = scalar([&]() { return sqrt(lo * hi); }, &one);
-        const double part = block_sum(sum(mid, false, chg), red);
-        if (threadIdx.x == 0) atomicAdd(a.sc + k % 3, part);
+    // Root of volume = target in u = log lam on the bracket [log 1e-12, log 1e12]: Newton steps, halving the
+    // bracket where a step leaves it, the slope vanishes or the step is not half the one before; done when
+    // a step is below 2e-10 or the bracket below 1e-9 (the bisection on the host ends at the latter). About
+    // eight sums where bisection takes 36. A volume that stays above (below) the target ends at the bracket's
+    // upper (lower) end, as there.
+    double lo = -27.631021115928547, hi = 27.631021115928547, u = 0.0, last = 1e300;
+    for (int k = 0; k < 200; ++k) {
+        const double li = scalar([&]() { return exp(-a.eta * u); }, &one);
+        double slope;
+        double part = sum(li, false, slope);
+        part = block_sum(part, red);
+        slope = block_sum(slope, red);
+        if (threadIdx.x == 0) {
+            atomicAdd(a.sc + 2 * (k % 3), part);
+            atomicAdd(a.sc + 2 * (k % 3) + 1, slope);
+        }
         if (!g.wait()) return;
-        const double tot = __ldcg(a.sc + k % 3);
-        // the sum of the step before is free again: nobody reads it past the barrier above
-        if (first == 0) __stcg(a.sc + (k + 2) % 3, 0.0);
-        if (tot > target) lo = mid;
-        else hi = mid;
+        const double f = __ldcg(a.sc + 2 * (k % 3)) - target, d = __ldcg(a.sc + 2 * (k % 3) + 1);
+        // the sums of the step before are free again: nobody reads them past the barrier above
+        if (first == 0) {
+            __stcg(a.sc + 2 * ((k + 2) % 3), 0.0);
+            __stcg(a.sc + 2 * ((k + 2) % 3) + 1, 0.0);
+        }
+        if (f > 0.0) lo = u;
+        else hi = u;
+        const double newton = scalar([&]() { return d < 0.0 ? u - f / d : 1e300; }, &one), move = fabs(newton - u);
+        const bool take = newton > lo && newton < hi && move < 0.5 * last;
+        const double to = take ? newton : 0.5 * (lo + hi);
+        last = take ? move : 1e300;
+        u = to;
+        if ((take && move < 2e-10) || hi - lo < 1e-9) break;
     }
-    const double vol = block_sum(sum(sqrt(lo * hi), true, chg), red);
+    double chg;
+    const double li = scalar([&]() { return exp(-a.eta * u); }, &one);
+    double vol = sum(li, true, chg);
+    vol = block_sum(vol, red);
     chg = block_sum(chg, red);
     if (threadIdx.x == 0) {
-        atomicAdd(a.sc + 5, vol);
-        atomicAdd(a.sc + 4, chg);
+        atomicAdd(a.sc + 8, vol);
+        atomicAdd(a.sc + 7, chg);
     }
 }
 

@@ -52,11 +52,10 @@ struct OcArgs {
     const float *xi, *S;
     const uint8_t *passive;
     double volfrac, move, eta, beta;
-    double li_lo, li_hi;                 // lam^-eta at the ends of the bracket of the multiplier
-    int steps;                           // bisection steps
     double *xs;                          // xi S^eta (n doubles of scratch)
     float *out;
-    double *sc;                          // [0..2] volume sums in turn, [3] count, [4] change, [5] final volume
+    double *sc;                          // [0..5] volume and slope sums, three pairs in turn, [6] count,
+                                         // [7] change, [8] final volume (zeroed before the launch)
     unsigned *bar;
 };
 cudaError_t oc_solve(const OcArgs &a, cudaStream_t s);

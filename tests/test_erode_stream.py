@@ -109,3 +109,29 @@ def test_streamed_minimum_equals_the_tiled_one(n, r, n_orient, groups):
         imf.close()
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,cut", [((64, 32), (3, 12)), ((65, 33), (1, 1)), ((7, 100), (5, 21)), ((200, 31), (9, 40)),
+                                   ((1, 1), (1, 2))])
+@pytest.mark.parametrize("groups", [0, 1])
+def test_planar_blocks_equal_the_3d_ones(n, cut, groups):
+    """One z-plane: the tiled minimum in planar blocks against the 3D blocks (erode_xt 8), at tile edges
+    and remainders: the minimum of the same values, so the same bits."""
+    torch = pytest.importorskip("torch")
+    from paper_2002_07627_gb300 import binding, build
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    tool = synth.planar_tool(cut[0], cut[1], cut[0] + 4, 6, n_orient=11)
+    rho = torch.rand((1, n[1], n[0]), generator=torch.Generator().manual_seed(1)).cuda()
+    got = []
+    for xt in (8, 0):
+        imf = binding.Imf(tuple(rho.shape), erode_xt=xt, erode_groups=groups)
+        imf.set_tool(0, tool.holder, tool.cutter, tool.origin, tool.quats)
+        raw = torch.empty_like(rho)
+        imf.compute(rho, raw=raw)
+        imf.sync()
+        got.append(raw.clone())
+        imf.close()
+    assert torch.equal(*got)
