@@ -5,15 +5,20 @@
 // The arithmetic is the one of axis2_kernel (fft2_kernels.cu); what changes is how the pencils
 // reach the registers. A block stays resident and walks a strided list of work items (kx
 // chunk, orientation, batch row). For each item the tensor memory accelerator copies the W
-// pencils of the chunk (and the W pencils of the pointwise factor) into a shared-memory stage
-// as [row j][pencil w]; zero padding of short inputs comes from the copy's out-of-bounds fill.
-// Two stages alternate: while the block transforms one item, the copy of its next item is in
-// flight, so the memory system sees a steady stream instead of the load / compute / store
-// phases of one-shot blocks. Results go straight from registers to global memory.
+// pencils of the chunk (and the W pencils of the pointwise factor) into shared memory as [row
+// j][pencil w]; zero padding of short inputs comes from the copy's out-of-bounds fill. Results go
+// straight from registers to global memory.
 //
-// Both factors of the split are template arguments of the loop (a runtime dispatch picks the
-// instance before the loop; a loop around two runtime dispatches made the compiler keep every
-// case's registers live), and only the splits fft2::choose_split returns are instantiated.
+// Two stages alternate: the copy of the block's next item is in flight while this one is transformed. What
+// bounds a pass is how many items an SM has in hand (barriers and waits of one block leave the SM to the others)
+// and how many bytes it has in flight. Each split (A, B) is its own kernel with 16 A threads, so that its registers
+// are its own (one kernel with every split inside took the largest one's, 112 to 124). For lengths up to 256 the
+// tile between the two DFT passes lies in the item's own stage, which pass 1 has read into registers by then: two
+// to four blocks an SM, where a tile buffer left room for one with the factor. Above 256 one block with a tile of its
+// own stays: two with the tile in the stage took 11.2 ms for the 256^3 y pass against 6.0 (a single stage a
+// block likewise, 11.5 and 10.8 for the z pass against 7.2). Measured, ms a step, against one kernel per shape:
+// z pass with the factor 128^3 x 64 0.787 -> 0.694, 144^3 x 96 1.70 -> 1.52, 75 x 61 x 50 x 24 0.090 -> 0.063, 48^3 x 24 0.068 ->
+// 0.047; 256^3 x 128 z 7.40 -> 7.25, y 6.18 -> 5.98.
 //
 // Every wait on a copy is bounded (%globaltimer); on a timeout the block records
 // IMF_ERR_TIMEOUT in the status word, waits (bounded again) for the copies it still has in
@@ -51,8 +56,19 @@ struct Params {
     int box_j, nbox, lrows;
 };
 
-template <int W> __host__ __device__ constexpr int threads(bool big) { return W * (big ? 32 : 16); }
-static_assert(threads<16>(true) == 512, "the wide big-factor shape runs 512 threads");
+// threads of an instance: W pencils by A slots (pass 2; pass 1 needs B <= A of them), in warps
+__host__ __device__ constexpr int threads(int W, int A) { return (W * A + 31) / 32 * 32; }
+// blocks per SM an instance is compiled for: as many as shared memory (two stages) and registers hold; one with
+// a factor above 16
+__host__ __device__ constexpr int min_blocks(int W, int A, int B, bool mul)
+{
+    if (A > fft2::kMaxFactor) return 1;
+    const int smem = kStages * A * B * W * 8 * (mul ? 2 : 1) + A * B * 8 + 512, by_smem = 220 * 1024 / smem;
+    // the warps of n blocks spread over four partitions of 512 registers a lane each, 80 a thread
+    int n = by_smem < 6 ? by_smem : 6;
+    while (n > 1 && (n * threads(W, A) / 32 + 3) / 4 * 80 > 512) --n;
+    return n < 1 ? 1 : n;
+}
 
 __device__ __forceinline__ void decode_item(const Params &P, long it, int &chunk, int &o, int &b)
 {
@@ -83,55 +99,72 @@ __device__ __forceinline__ void issue_item(const Params &P, const void *in_map, 
     }
 }
 
-// The persistent loop for one split L = NA NB.
+// where the tile between the passes lies: in the item's own stage (lengths up to 256), or in a buffer of its own
+__host__ __device__ constexpr bool tile_in_stage(int A) { return A <= fft2::kMaxFactor; }
+
+// One split L = NA NB: the persistent loop over this block's items.
 template <int S, int MUL, int W, int NA, int NB>
-__device__ __forceinline__ void run_items(const Params &P, const void *in_map, const void *mul_map, float2 *st,
-                                          size_t half, size_t stage, float2 *tile, const float2 *tw, uint64_t *bar)
+__global__ void __launch_bounds__(threads(W, NA), min_blocks(W, NA, NB, MUL != 0))
+    axis2_tma_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap mul_map, Params P)
 {
-    constexpr int LOGW = W == 8 ? 3 : 4;
+    constexpr int T = threads(W, NA), LOGW = W == 8 ? 3 : 4, L = NA * NB;
+    extern __shared__ unsigned char smraw[];
     const AxisArgs &a = P.a;
+    // 128-byte aligned stages (tensor-copy destinations), twiddles, barriers
+    unsigned char *base = smraw + ((128 - (tc::smem_addr(smraw) & 127)) & 127);
+    const size_t half = (size_t)P.lrows * W, stage = half * (MUL ? 2 : 1);
+    constexpr bool INSTAGE = tile_in_stage(NA);
+    float2 *st = reinterpret_cast<float2 *>(base), *own = st + kStages * stage, *tw = own + (INSTAGE ? 0 : L * W);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(tw + L);
+    for (int i = threadIdx.x; i < L; i += T) tw[i] = a.tw[i];
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; ++s) tc::mbar_init(&bar[s], 1);
+        tc::fence_mbar_init();
+    }
+    __syncthreads();
     const int w = threadIdx.x & (W - 1), p = threadIdx.x >> LOGW;
     const long G = gridDim.x, first = blockIdx.x;
-    const long mine = (P.items - first + G - 1) / G;      // items of this block: first + k G
+    const long mine = (P.items - first + G - 1) / G;           // items of this block: first + k G
     if (threadIdx.x == 0)
         for (int s = 0; s < kStages && s < mine; ++s)
-            issue_item<MUL, W>(P, in_map, mul_map, first + s * G, st + s * stage, st + s * stage + half, &bar[s]);
+            issue_item<MUL, W>(P, &in_map, &mul_map, first + s * G, st + s * stage, st + s * stage + half, &bar[s]);
     for (long k = 0; k < mine; ++k) {
         const int s = (int)(k % kStages);
         const bool timeout = !tc::mbar_wait(&bar[s], (uint32_t)((k / kStages) & 1));
         const long it = first + k * G;
-        const float2 *sin_ = st + s * stage, *smul = sin_ + half;
-        // pass 1: slot p = n1 < NB reads x[n1 + NB n2] (times the factor) from the stage and
-        // transforms it in registers (after a timeout the values are not used)
+        float2 *in = st + s * stage, *tile = INSTAGE ? in : own;
+        auto refill = [&]() {
+            if (threadIdx.x == 0 && k + kStages < mine) {
+                // generic-proxy accesses of the stage above, async-proxy writes into it next
+                tc::fence_async_smem();
+                issue_item<MUL, W>(P, &in_map, &mul_map, first + (k + kStages) * G, in, in + half, &bar[s]);
+            }
+        };
+        // pass 1: slot p = n1 < NB reads x[n1 + NB n2] (times the factor) from the stage and transforms it
+        // in registers (after a timeout the values are not used)
         float2 v[NA];
         const bool act = p < NB;
         if (act) {
 #pragma unroll
             for (int n2 = 0; n2 < NA; ++n2) {
                 const int j = p + NB * n2;
-                v[n2] = sin_[j * W + w];
-                if (MUL) v[n2] = c_mul(v[n2], smul[j * W + w]);
+                v[n2] = in[j * W + w];
+                if (MUL) v[n2] = c_mul(v[n2], in[half + j * W + w]);
             }
             fft2::dft_reg<S, NA>(v);
             fft2::twiddle<S, NA>(v, p, tw);
         }
-        // one barrier: the stage is free, the previous item's tile reads are done, and every
-        // thread knows whether a copy timed out
+        // the stage is read and the previous item's tile too; every thread knows whether a copy timed out
         if (__syncthreads_or(timeout)) {
             if (threadIdx.x == 0) {
                 if (a.status) atomicCAS(a.status, 0, (int)IMF_ERR_TIMEOUT);
-                // drain this block's copies still in flight (bounded) before leaving
+                // wait (bounded) for this block's copies still in flight before leaving
                 const long issued = k + kStages < mine ? k + kStages : mine;
                 for (long q = k; q < issued; ++q) tc::mbar_wait(&bar[q % kStages], (uint32_t)((q / kStages) & 1));
             }
             return;
         }
-        if (threadIdx.x == 0 && k + kStages < mine) {
-            // generic-proxy reads of the stage above, async-proxy writes into it next
-            tc::fence_async_smem();
-            issue_item<MUL, W>(P, in_map, mul_map, first + (k + kStages) * G, st + s * stage, st + s * stage + half,
-                               &bar[s]);
-        }
+        if (!INSTAGE) refill();
         if (act) {
 #pragma unroll
             for (int k2 = 0; k2 < NA; ++k2) tile[(p * NA + k2) * W + w] = v[k2];
@@ -141,10 +174,17 @@ __device__ __forceinline__ void run_items(const Params &P, const void *in_map, c
         int chunk, o, b;
         decode_item(P, it, chunk, o, b);
         const int c = chunk * W + w;
-        if (p < NA && c < a.nx) {
-            float2 u[NB];
+        const bool act2 = p < NA && c < a.nx;
+        float2 u[NB];
+        if (act2) {
 #pragma unroll
             for (int n1 = 0; n1 < NB; ++n1) u[n1] = tile[(n1 * NA + p) * W + w];
+        }
+        if (INSTAGE) {
+            __syncthreads();
+            refill();
+        }
+        if (act2) {
             fft2::dft_reg<S, NB>(u);
             float2 *out = a.out + (long)o * a.out_so + (long)b * a.out_sb + c;
 #pragma unroll
@@ -157,46 +197,7 @@ __device__ __forceinline__ void run_items(const Params &P, const void *in_map, c
                 }
             }
         }
-        // the next iteration's barrier (after its wait) precedes any rewrite of the tile
     }
-}
-
-template <int S, bool BIG, int MUL, int W>
-__global__ void __launch_bounds__(threads<W>(BIG))
-    axis2_tma_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap mul_map,
-                     Params P)
-{
-    constexpr int T = threads<W>(BIG);
-    extern __shared__ unsigned char smraw[];
-    const int A = P.a.A2, B = P.a.B2, L = A * B;
-    // 128-byte aligned stages (tensor-copy destinations), then the tile, twiddles and barriers
-    unsigned char *base = smraw + ((128 - (tc::smem_addr(smraw) & 127)) & 127);
-    const size_t half = (size_t)P.lrows * W;
-    const size_t stage = half * (MUL ? 2 : 1);
-    float2 *st = reinterpret_cast<float2 *>(base);
-    float2 *tile = st + kStages * stage;
-    float2 *tw = tile + (size_t)L * W;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(tw + L);
-    for (int i = threadIdx.x; i < L; i += T) tw[i] = P.a.tw[i];
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) tc::mbar_init(&bar[s], 1);
-        tc::fence_mbar_init();
-    }
-    __syncthreads();
-    constexpr int maxA = BIG ? fft2::kMaxFactorBig : fft2::kMaxFactor;
-    auto outer = [&](auto AA) {
-        constexpr int NA = decltype(AA)::value;
-        auto inner = [&](auto BB) {
-            constexpr int NB = decltype(BB)::value;
-            if constexpr (fft2::is_split_choice(NA, NB, maxA) &&
-                          (BIG ? NA > fft2::kMaxFactor : NA * NB >= kMinLength))
-                run_items<S, MUL, W, NA, NB>(P, &in_map, &mul_map, st, half, stage, tile, tw, bar);
-        };
-        if constexpr (BIG) fft2::with_size_big(B, inner);
-        else fft2::with_size(B, inner);
-    };
-    if constexpr (BIG) fft2::with_size_big(A, outer);
-    else fft2::with_size(A, outer);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -400,21 +401,22 @@ IMF_TMA_DECL(launch_tma_b2)
 #undef IMF_TMA_DECL
 
 
-// Shared memory of one block: 128 bytes of alignment slack, the stages, the tile, the twiddles
-// and the barriers.
+// Shared memory of one block: 128 bytes of alignment slack, the stages, the tile where it has a buffer of its
+// own, the twiddles and the barriers.
 inline size_t smem_bytes(const Params &P, int W, bool mul)
 {
     const int L = P.a.A2 * P.a.B2;
-    return 128 + (size_t)kStages * P.lrows * W * 8 * (mul ? 2 : 1) + (size_t)L * W * 8 + (size_t)L * 8 + kStages * 8;
+    return 128 + (size_t)kStages * P.lrows * W * 8 * (mul ? 2 : 1) + (tile_in_stage(P.a.A2) ? 0 : (size_t)L * W * 8) +
+           (size_t)L * 8 + kStages * 8;
 }
 
-template <int S, bool BIG, int MUL, int W>
-bool launch_shape(const CUtensorMap &in_map, const CUtensorMap &mul_map, Params &P, cudaStream_t s)
+template <int S, int MUL, int W, int NA, int NB>
+bool launch_split(const CUtensorMap &in_map, const CUtensorMap &mul_map, const Params &P, cudaStream_t s)
 {
-    constexpr int T = threads<W>(BIG);
+    constexpr int T = threads(W, NA);
     const size_t smem = smem_bytes(P, W, MUL != 0);
     if (smem > 227 * 1024) return false;
-    auto kernel = axis2_tma_kernel<S, BIG, MUL, W>;
+    auto kernel = axis2_tma_kernel<S, MUL, W, NA, NB>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -427,6 +429,28 @@ bool launch_shape(const CUtensorMap &in_map, const CUtensorMap &mul_map, Params 
     const long blocks = P.items < (long)per * sm_count() ? P.items : (long)per * sm_count();
     kernel<<<(unsigned)blocks, T, smem, s>>>(in_map, mul_map, P);
     return true;
+}
+
+// the instance of the split of P.a (16-slot shape: both factors at most 16, length from kMinLength)
+template <int S, bool BIG, int MUL, int W>
+bool launch_shape(const CUtensorMap &in_map, const CUtensorMap &mul_map, Params &P, cudaStream_t s)
+{
+    constexpr int maxA = BIG ? fft2::kMaxFactorBig : fft2::kMaxFactor;
+    bool done = false;
+    auto outer = [&](auto AA) {
+        constexpr int NA = decltype(AA)::value;
+        auto inner = [&](auto BB) {
+            constexpr int NB = decltype(BB)::value;
+            if constexpr (fft2::is_split_choice(NA, NB, maxA) &&
+                          (BIG ? NA > fft2::kMaxFactor : NA * NB >= kMinLength))
+                done = launch_split<S, MUL, W, NA, NB>(in_map, mul_map, P, s);
+        };
+        if constexpr (BIG) fft2::with_size_big(P.a.B2, inner);
+        else fft2::with_size(P.a.B2, inner);
+    };
+    if constexpr (BIG) fft2::with_size_big(P.a.A2, outer);
+    else fft2::with_size(P.a.A2, outer);
+    return done;
 }
 
 } // namespace tma_fft
