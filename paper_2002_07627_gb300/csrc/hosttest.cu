@@ -12,6 +12,7 @@
 #include "fft_plan.h"
 #include "orient_order.h"
 #include "sweep_bits.cuh"
+#include "sweep_plan.h"
 
 extern "C" int imf_host_fft(int L, int sign, const float *in, float *out)
 {
@@ -168,6 +169,24 @@ extern "C" int imf_host_plan_stream(const int *sh, int n_pts, const int *K, int 
                          h[0].axis, h[0].lists, h[0].rows, h[0].quads, h[0].ox, h[0].ou, h[0].ow};
     std::memcpy(head, out, sizeof out);
     if ((int)words.size() > max_words || h[0].words != (int)words.size() || g.words != h[0].words) return -2;
+    std::memcpy(words_out, words.data(), words.size() * sizeof(int));
+    return (int)words.size();
+}
+
+// The plan of the sweep on staged tiles (sweep_plan.h) of one orientation's cutter offsets. head gets nq, nl,
+// planes per warp, row pitch, largest word shift, planes staged, bytes, axis, eu, ew, ou, ow; words the descriptors.
+// Returns the number of words, -1 where the plan refuses the cutter and -2 when the output array is too small.
+extern "C" int imf_host_plan_sweep(const int *rk, int n_pts, const int *K, const int *kmin, int nx, int *head, int max_words,
+                                   int *words_out)
+{
+    std::vector<std::vector<int32_t>> v(1, std::vector<int32_t>(rk, rk + 3 * (size_t)n_pts));
+    std::vector<imf::SwOrient> h;
+    std::vector<int> words;
+    imf::SwGeometry g;
+    if (!imf::sw_plan(v, K, kmin, nx, g, h, words)) return -1;
+    const int out[12] = {g.nq, g.nl, g.ppw, g.UP, g.somax, g.planes, (int)g.smem, h[0].axis, h[0].eu, h[0].ew, h[0].ou, h[0].ow};
+    std::memcpy(head, out, sizeof out);
+    if ((int)words.size() > max_words || h[0].words != (int)words.size()) return -2;
     std::memcpy(words_out, words.data(), words.size() * sizeof(int));
     return (int)words.size();
 }

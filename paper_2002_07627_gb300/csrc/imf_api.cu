@@ -30,6 +30,7 @@
 #include "erode_stream.h"
 #include "fft_plan.h"
 #include "orient_order.h"
+#include "sweep_plan.h"
 
 using namespace imf;
 
@@ -81,6 +82,10 @@ struct Tool {
     int *rt_start = nullptr;
     int4 *sw_pairs = nullptr;            // sweep run descriptors (SweepArgs::pairs), all orientations
     int *sw_start = nullptr;
+    bool sw_ok = false;                  // planned for the sweep on staged tiles (sweep_tile.cu)
+    SwGeometry sw;
+    SwOrient *sw_head = nullptr;
+    int *sw_words = nullptr;
     ErodeChunk *er_chunks = nullptr;
     int *er_chunk_start = nullptr;
     int2 *er_runs = nullptr;
@@ -421,6 +426,8 @@ void free_tool(imf_handle h, Tool &t)
     dfree(h, t.rt_start, (size_t)t.n_orient + 1);
     dfree(h, t.sw_pairs, (size_t)0);
     dfree(h, t.sw_start, (size_t)t.n_orient + 1);
+    dfree(h, t.sw_head);
+    dfree(h, t.sw_words);
     dfree(h, t.er_chunks);
     dfree(h, t.er_chunk_start);
     dfree(h, t.er_runs);
@@ -1160,6 +1167,10 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
     if (!t.es_ok) { es_head.clear(); es_words.clear(); }
     t.es_axis.clear();
     for (const EsOrient &e : es_head) t.es_axis.push_back((signed char)e.axis);
+    std::vector<SwOrient> sw_head;
+    std::vector<int> sw_words;
+    t.sw_ok = sw_plan(t.rk, t.kmax, t.kmin, h->opt.nx, t.sw, sw_head, sw_words);
+    if (!t.sw_ok) { sw_head.clear(); sw_words.clear(); }
     if (!plan_only) {
         int dev = 0, n = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -1177,7 +1188,8 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
                     vbytes(ivv.size(), sizeof(int4)) + vbytes(ivst.size(), 4) +
                     vbytes(chunks.size(), sizeof(ErodeChunk)) + vbytes(chst.size(), 4) +
                     vbytes(eruns.size(), sizeof(int2)) + vbytes(t.perm.size(), 4) +
-                    vbytes(es_head.size(), sizeof(EsOrient)) + vbytes(es_words.size(), 4);
+                    vbytes(es_head.size(), sizeof(EsOrient)) + vbytes(es_words.size(), 4) +
+                    vbytes(sw_head.size(), sizeof(SwOrient)) + vbytes(sw_words.size(), 4);
     if (!plan_only) {
         twiddles(t.M, t.M, t.M, tw);
         if ((st = upload(h, &t.twM, tw))) return bail(st);
@@ -1191,7 +1203,8 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
             (st = upload(h, &t.sw_pairs, ivv)) || (st = upload(h, &t.sw_start, ivst)) ||
             (st = upload(h, &t.er_chunks, chunks)) || (st = upload(h, &t.er_chunk_start, chst)) ||
             (st = upload(h, &t.er_runs, eruns)) || (st = upload(h, &t.perm_dev, t.perm)) ||
-            (st = upload(h, &t.es_head, es_head)) || (st = upload(h, &t.es_words, es_words)))
+            (st = upload(h, &t.es_head, es_head)) || (st = upload(h, &t.es_words, es_words)) ||
+            (st = upload(h, &t.sw_head, sw_head)) || (st = upload(h, &t.sw_words, sw_words)))
             return bail(st);
     }
     // --- direct tensor-core path: groups, union taps, B matrices
@@ -1273,7 +1286,21 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         Launch L(h, KID_RECHECK, s);
         launch_recheck_blocks(a, 152 * 64, s);     // up to 64 points (warps) in flight per SM
     }
-    if (h->run_sweep) {
+    if (h->run_sweep && t.sw_ok && !op.sweep_loop) {
+        SwArgs a{};
+        a.bits = h->bits; a.b_so = bso; a.wpr = t.wpr; a.wy = t.win[1]; a.wz = t.win[2];
+        a.head = t.sw_head; a.words = t.sw_words; a.nx = op.nx; a.ny = op.ny; a.nz = op.nz;
+        a.awords = h->awords; a.orient_base = o0; a.nb = nb; a.A = h->A; a.geo = t.sw;
+        if (h->aset) {
+            long base = 0;
+            for (int i = 0; i < h->n_tools && &h->tools[i] != &t; ++i) base += h->tools[i].n_orient;
+            a.A_per = h->aset + base * h->aset_so;
+            a.a_per_so = h->aset_so;
+            a.perm = t.perm_dev;
+        }
+        Launch L(h, KID_SWEEP, s);
+        launch_sweep_tile(a, s);
+    } else if (h->run_sweep) {
         const long lstride = (long)h->bits_n * h->slots;
         {
             SweepLevelsArgs a{};
