@@ -245,6 +245,10 @@ __global__ void __launch_bounds__(kT2) irfft2_threshold_kernel(IrfftArgs a)
 //     n1 A + k2 of the row itself (A B = M <= hs); pass 2 ends in the threshold epilogue.
 // Each pass loops inside one size case of the uniform dispatch (a loop around the dispatch
 // would keep every case's registers live); the free-bit words are packed at the end.
+// NT threads: 512 (32 columns by 16 slots) where the plane leaves room for one block an SM, 256 (16 by 16) where
+// two fit, so that the copy and the barriers of one overlap the transforms of the other (512 threads of the
+// registers this kernel takes fill an SM). us a step, 512 -> 256 threads: 48^3 x 24 100 -> 84, 75 x 61 x 50 x 24
+// 136 -> 108, 96^3 x 32 350 -> 286.
 constexpr int kYX = 512;
 
 __host__ __device__ inline long yx2_flags_offset(int Ly, int hs, int M)
@@ -252,8 +256,9 @@ __host__ __device__ inline long yx2_flags_offset(int Ly, int hs, int M)
     return ((long)Ly * hs + Ly + 2 * M + 1 + 1) & ~1L;   // float2 offset, 16-byte aligned
 }
 
-__global__ void __launch_bounds__(kYX) yx2_threshold_kernel(AxisArgs ay, IrfftArgs a, int hs)
+template <int NT> __global__ void __launch_bounds__(NT, kYX / NT) yx2_threshold_kernel(AxisArgs ay, IrfftArgs a, int hs)
 {
+    constexpr int CG = NT / 16;                // columns of a group
     extern __shared__ float2 sm[];
     __shared__ uint64_t bar;
     const int Ay = ay.A2, By = ay.B2, Ly = Ay * By, Hx = ay.nx;
@@ -270,9 +275,9 @@ __global__ void __launch_bounds__(kYX) yx2_threshold_kernel(AxisArgs ay, IrfftAr
         tc::mbar_expect_tx(&bar, bytes);
         tc::bulk_g2s(plane, ay.in + o * ay.in_so + (long)z * ay.in_sb, bytes, &bar);
     }
-    for (int i = threadIdx.x; i < Ly; i += kYX) twy[i] = ay.tw[i];
-    for (int i = threadIdx.x; i < M; i += kYX) twM[i] = a.twM[i];
-    for (int i = threadIdx.x; i <= M; i += kYX) twP[i] = a.twP[i];
+    for (int i = threadIdx.x; i < Ly; i += NT) twy[i] = ay.tw[i];
+    for (int i = threadIdx.x; i < M; i += NT) twM[i] = a.twM[i];
+    for (int i = threadIdx.x; i <= M; i += NT) twP[i] = a.twP[i];
     __syncthreads();
     if (!tc::mbar_wait(&bar, 0)) {
         // the copy did not land in time: report it, give it one more bounded wait, stop
@@ -280,55 +285,55 @@ __global__ void __launch_bounds__(kYX) yx2_threshold_kernel(AxisArgs ay, IrfftAr
         tc::mbar_wait(&bar, 0);
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // y pass 1: slot p = warp < By loads x[p + By n2] of column c, A-point DFT and twiddles,
+    const int lane = threadIdx.x & 31, col = threadIdx.x % CG, slot = threadIdx.x / CG;
+    // y pass 1: slot p < By loads x[p + By n2] of column c, A-point DFT and twiddles,
     // element (n1, k2) back to row n1 Ay + k2 of the column
     fft2::with_size(Ay, [&](auto AA) {
         constexpr int NA = decltype(AA)::value;
-        for (int c0 = 0; c0 < Hx; c0 += 32) {
-            const int c = c0 + lane;
-            const bool act = warp < By && c < Hx;
+        for (int c0 = 0; c0 < Hx; c0 += CG) {
+            const int c = c0 + col;
+            const bool act = slot < By && c < Hx;
             float2 v[NA];
             if (act) {
 #pragma unroll
-                for (int n2 = 0; n2 < NA; ++n2) v[n2] = plane[(long)(warp + By * n2) * hs + c];
-                fft2::pass1<1, NA>(v, warp, twy);
+                for (int n2 = 0; n2 < NA; ++n2) v[n2] = plane[(long)(slot + By * n2) * hs + c];
+                fft2::pass1<1, NA>(v, slot, twy);
             }
             __syncthreads();
             if (act) {
 #pragma unroll
-                for (int k2 = 0; k2 < NA; ++k2) plane[(long)(warp * NA + k2) * hs + c] = v[k2];
+                for (int k2 = 0; k2 < NA; ++k2) plane[(long)(slot * NA + k2) * hs + c] = v[k2];
             }
         }
     });
     __syncthreads();
-    // y pass 2: slot p = warp < Ay, By-point DFT over n1, X[p + Ay k1] to row p + Ay k1 < lout
+    // y pass 2: slot p = slot < Ay, By-point DFT over n1, X[p + Ay k1] to row p + Ay k1 < lout
     fft2::with_size(By, [&](auto BB) {
         constexpr int NB = decltype(BB)::value;
-        for (int c0 = 0; c0 < Hx; c0 += 32) {
-            const int c = c0 + lane;
-            const bool act = warp < Ay && c < Hx;
+        for (int c0 = 0; c0 < Hx; c0 += CG) {
+            const int c = c0 + col;
+            const bool act = slot < Ay && c < Hx;
             float2 u[NB];
             if (act) {
 #pragma unroll
-                for (int n1 = 0; n1 < NB; ++n1) u[n1] = plane[(long)(n1 * Ay + warp) * hs + c];
+                for (int n1 = 0; n1 < NB; ++n1) u[n1] = plane[(long)(n1 * Ay + slot) * hs + c];
                 fft2::dft_reg<1, NB>(u);
             }
             __syncthreads();
             if (act) {
 #pragma unroll
                 for (int k1 = 0; k1 < NB; ++k1) {
-                    const int y = warp + Ay * k1;
+                    const int y = slot + Ay * k1;
                     if (y < ay.lout) plane[(long)y * hs + c] = u[k1];
                 }
             }
         }
     });
     __syncthreads();
-    // x pass 1: rows of Bx threads, kYX / Bx rows per round
+    // x pass 1: rows of Bx threads, NT / Bx rows per round
     fft2::with_size(Ax, [&](auto AA) {
         constexpr int NA = decltype(AA)::value;
-        const int w0 = threadIdx.x / Bx, p = threadIdx.x - w0 * Bx, rpr = kYX / Bx;
+        const int w0 = threadIdx.x / Bx, p = threadIdx.x - w0 * Bx, rpr = NT / Bx;
         for (int y0 = 0; y0 < nrow; y0 += rpr) {
             const int y = y0 + w0;
             const bool act = w0 < rpr && y < nrow;
@@ -345,10 +350,10 @@ __global__ void __launch_bounds__(kYX) yx2_threshold_kernel(AxisArgs ay, IrfftAr
         }
     });
     __syncthreads();
-    // x pass 2 and the threshold epilogue: rows of Ax threads, kYX / Ax rows per round
+    // x pass 2 and the threshold epilogue: rows of Ax threads, NT / Ax rows per round
     fft2::with_size(Bx, [&](auto BB) {
         constexpr int NB = decltype(BB)::value;
-        const int w0 = threadIdx.x / Ax, p = threadIdx.x - w0 * Ax, rpr = kYX / Ax;
+        const int w0 = threadIdx.x / Ax, p = threadIdx.x - w0 * Ax, rpr = NT / Ax;
         for (int y0 = 0; y0 < nrow; y0 += rpr) {
             const int y = y0 + w0;
             const bool act = w0 < rpr && y < nrow;
@@ -363,7 +368,7 @@ __global__ void __launch_bounds__(kYX) yx2_threshold_kernel(AxisArgs ay, IrfftAr
     });
     if (!a.write_bits) return;   // uniform
     __syncthreads();
-    x_pack_bits<kYX>(a, sflag, fp, z * nrow, nrow, o);
+    x_pack_bits<NT>(a, sflag, fp, z * nrow, nrow, o);
 }
 
 template <typename K> void set_smem2(K kernel, size_t bytes)
@@ -453,9 +458,16 @@ bool yx2_fits(const AxisArgs &ay, const IrfftArgs &a, int hs)
 
 void launch_yx2_threshold(const AxisArgs &ay, const IrfftArgs &a, int hs, int nz, int norient, cudaStream_t s)
 {
-    const size_t smem = yx2_smem(ay.A2 * ay.B2, hs, a.M, a.rows_y);
-    set_smem2(yx2_threshold_kernel, smem);
-    yx2_threshold_kernel<<<dim3(nz, norient), kYX, smem, s>>>(ay, a, hs);
+    // the flag bytes are there only where the free bits are stored
+    const size_t smem = yx2_smem(ay.A2 * ay.B2, hs, a.M, a.write_bits ? a.rows_y : 0);
+    const dim3 grid(nz, norient);
+    if (2 * (smem + 1024 + 64) <= 228 * 1024) {
+        set_smem2(yx2_threshold_kernel<kYX / 2>, smem);
+        yx2_threshold_kernel<kYX / 2><<<grid, kYX / 2, smem, s>>>(ay, a, hs);
+    } else {
+        set_smem2(yx2_threshold_kernel<kYX>, smem);
+        yx2_threshold_kernel<kYX><<<grid, kYX, smem, s>>>(ay, a, hs);
+    }
 }
 
 } // namespace imf
