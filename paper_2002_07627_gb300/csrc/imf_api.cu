@@ -1516,7 +1516,7 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
             h->last_tool = ti;
         }
     }
-    {
+    if (!small_grid(N)) {
         Launch L(h, KID_MAX, s);
         launch_max_omega0(h->f, fix, N, maxbits, s);
     }
@@ -1527,7 +1527,8 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
         a.fbar = fbar; a.secluded = sec; a.raw = raw; a.acc = acc;
         a.acc_from_f = acc_from_f; a.theta = (float)h->tools[0].theta;
         Launch L(h, KID_FINALIZE, s);
-        launch_finalize(a, s);
+        if (small_grid(N)) launch_finalize_small(a, s);
+        else launch_finalize(a, s);
     }
     CU(cudaGetLastError());
     h->computes++;
@@ -1587,11 +1588,15 @@ imf_status imf_penalize_sensitivity(imf_handle h, float *sens, const float *rho_
     h->last_stream = s;
     h->used_stream = true;
     // the maximum's word is zero between calls: allocated so, and cleared by the kernel that reads it
-    {
-        Launch L(h, KID_ABSMAX, s);
-        launch_absmax_omega0(sens, fixture, N, mb, s);
-    }
-    {
+    if (small_grid(N)) {
+        Launch L(h, KID_PENALIZE, s);
+        launch_penalize_small(sens, rho_omega, imf_bar, secluded, fixture, N, mb, (unsigned *)(h->dev_small + 5), w_acc,
+                              h->opt.tau, s);
+    } else {
+        {
+            Launch L(h, KID_ABSMAX, s);
+            launch_absmax_omega0(sens, fixture, N, mb, s);
+        }
         Launch L(h, KID_PENALIZE, s);
         launch_penalize(sens, rho_omega, imf_bar, secluded, N, mb, (unsigned *)(h->dev_small + 5), w_acc, h->opt.tau, s);
     }

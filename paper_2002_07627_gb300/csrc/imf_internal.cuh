@@ -243,7 +243,7 @@ struct FinalizeArgs {
     const uint8_t *fix;
     const uint32_t *A;
     int nx, ny, nz, awords;
-    const unsigned *maxbits;
+    unsigned *maxbits;
     double lambda, tau;
     float *fbar;
     uint8_t *secluded;
@@ -253,6 +253,11 @@ struct FinalizeArgs {
     float theta;
 };
 void launch_finalize(const FinalizeArgs &a, cudaStream_t s);
+// grids small enough for the two below: the maximum over Omega_0 and what follows from it in one launch
+bool small_grid(long n);
+void launch_finalize_small(const FinalizeArgs &a, cudaStream_t s);
+void launch_penalize_small(float *sens, const float *rho, const float *fbar, const uint8_t *sec, const uint8_t *fix, long n,
+                           unsigned *maxbits, unsigned *done, double w, double tau, cudaStream_t s);
 void launch_absmax_omega0(const float *v, const uint8_t *fix, long n, unsigned *maxbits, cudaStream_t s);
 void launch_penalize(float *sens, const float *rho, const float *fbar, const uint8_t *sec, long n,
                      unsigned *maxbits, unsigned *done, double w, double tau, cudaStream_t s);

@@ -125,3 +125,39 @@ def test_greedy_plan_matches_the_oracle_on_given_sets(shape, n_sets, max_steps):
     want = oracle.process_plan(list(sets), (fix == 0) & (rho <= 0.5), max_steps)
     assert (steps, neg, left) == want
     imf.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (1, 7, 31), (1, 128, 256), (1, 129, 256), (2, 3, 5)])
+@pytest.mark.parametrize("fixture", [False, True])
+def test_normalisation_and_penalty_around_the_small_grid_limit(shape, fixture):
+    """32768 voxels run the maximum and what follows from it in one cluster, more of them in two launches:
+    f_bar and Gamma from the raw f by the FP64 formula (whole values equal, f_bar to its last FP32 bit), and
+    the penalty twice in a row (its maximum starts from zero again), against NumPy."""
+    binding = _need()
+    from paper_2002_07627_gb300 import synth
+    rng = np.random.default_rng(shape[2])
+    rho = rng.uniform(0, 1, shape).astype(np.float32)
+    fix = (rng.uniform(size=shape) < 0.2).astype(np.uint8) if fixture else None
+    tool = synth.planar_tool(1, 2, 3, 2, n_orient=3)
+    imf = binding.Imf(shape)
+    imf.set_tools([tool])
+    r, f = _dev(rho), None if fix is None else _dev(fix)
+    raw = torch.empty_like(r)
+    fbar, sec = imf.compute(r, f, raw=raw)
+    imf.sync()
+    g = raw.cpu().numpy().astype(np.float64)
+    omega = np.ones(shape, bool) if fix is None else fix == 0
+    M = g[omega].max() if omega.any() else 0.0
+    fb = np.where(omega, g * (1.0 / M) if M > 0 else 0.0, 0.0)
+    B = fb > 0.01
+    want = (fb * B).astype(np.float32)
+    assert np.abs(fbar.cpu().numpy() - want).max() <= np.spacing(np.float32(1.0))
+    assert np.array_equal(sec.cpu().numpy(), (omega & (rho <= 0.5) & B).astype(np.uint8))
+    for scale in (3.0, 0.25):
+        s0 = (rng.standard_normal(shape) * scale).astype(np.float32)
+        out = imf.penalize(_dev(s0), r, fbar, sec, f, w_acc=0.3).cpu().numpy().astype(np.float64)
+        m = np.abs(s0[omega]).max() if omega.any() else 0.0
+        s_imf = np.where(rho > 0.5, want, np.where(omega & (rho <= 0.5) & B, 1.0, 0.0))
+        ref = 0.7 * (s0 / m if m > 0 else s0) + 0.3 * s_imf
+        assert np.abs(out - ref).max() <= 4e-7 * max(1.0, np.abs(ref).max())
+    imf.close()
