@@ -16,6 +16,9 @@
 // finish early) does not leave SMs idle at the end. Groups of one tile then merge into f with
 // an integer atomic minimum, which orders non-negative floats (every g >= 0; -0 is mapped to +0
 // first) exactly as the float minimum does, so the result does not depend on the split.
+//
+// Large 3D grids take erode_stream.cu instead (imf_api.cu holds the rule); this kernel serves planar grids,
+// grids of few tiles, where it is as fast or faster, and the forms that the options choose.
 #include <cfloat>
 
 #include "erode.cuh"
