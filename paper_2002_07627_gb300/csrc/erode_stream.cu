@@ -24,8 +24,9 @@
 // Against the tiled kernel (ms per step): 256^3 x 128 43.5 -> 34.1, 128^3 x 64 2.98 -> 2.47, 144^3 x 96 with a
 // radius-6 cutter 17.2 -> 13.5.
 //
-// Every wait is bounded; on a timeout the block records IMF_ERR_TIMEOUT, its producers wait for their own
-// copies, and it leaves.
+// Every wait on a stage is bounded; on a timeout the block records IMF_ERR_TIMEOUT and leaves, its producers
+// together (es_produce) and after the copies they issued have landed. The two named barriers need no limit:
+// all that they count reach them, since every wait before them ends.
 #include "erode_stream.cuh"
 #include "imf.h"
 #include "imf_internal.cuh"
@@ -189,6 +190,95 @@ __device__ __forceinline__ void copies_arrive(uint64_t *bar)
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(tc::smem_addr(bar)) : "memory");
 }
 
+// whether `p` holds in any of the producers; a barrier of all of them
+__device__ __forceinline__ bool any_producer(bool p)
+{
+    uint32_t r;
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+                 : "=r"(r)
+                 : "r"((uint32_t)p), "n"(kEsProducers)
+                 : "memory");
+    return r != 0;
+}
+
+// A producer thread: copies the planes of every orientation of its block's kind into the ring (es_produce).
+template <int P> struct EsProducer {
+    const EsArgs &a;
+    const unsigned short *s_ob;
+    int *s_words;
+    unsigned char *s_live, (*s_list)[32], (*s_off)[kEsNW + 1];
+    uint64_t *full, *empty;
+    int *s_stop;
+    uint32_t ring0, stage_bytes;
+    int axis, X0, U0, W0;
+    // the orientation it is at
+    EsOrient h;
+    int ob, cols, rows, gu0;
+    const float *src0;
+
+    __device__ __forceinline__ int steps(int k)
+    {
+        ob = s_ob[k];
+        h = a.head[a.orient_base + ob];
+        gu0 = U0 + h.ou;
+        cols = min(h.quads, (a.gpx - (X0 + h.ox)) >> 2);       // columns the window's rows have from here
+        rows = min(h.rows, (axis ? a.wz : a.wy) - gu0);
+        src0 = a.g + ob * a.g_so + X0 + h.ox;
+        return kEsNW + h.lists;
+    }
+    __device__ __forceinline__ bool wait(int st, uint32_t phase)
+    {
+        if (tc::mbar_wait(&empty[st], phase)) return true;
+        if (a.status) atomicCAS(a.status, 0, (int)IMF_ERR_TIMEOUT);
+        return false;
+    }
+    __device__ __forceinline__ EsOpen open(int k, int st, bool late)
+    {
+        const int tid = threadIdx.x - 32 * kEsWarps, lane = tid & 31, slot = k % kEsSlots;
+        // the orientation's descriptors; the slot's last readers, four orientations back, gave
+        // back their stages at least ten stages ago (an orientation has three or more)
+        if (!late)
+            for (int i = tid; i < h.words / 4; i += kEsProducers)
+                reinterpret_cast<int4 *>(s_words + slot * a.geo.words)[i] = __ldg(reinterpret_cast<const int4 *>(a.words + h.word0) + i);
+        // the units that still have work, as one warp sees them; none: the block is done
+        if (tid < 32) {
+            const uint32_t mask = __ballot_sync(0xffffffffu, ((volatile unsigned char *)s_live)[lane] != 0);
+            if (!late) {
+                if (mask >> lane & 1) s_list[slot][__popc(mask & ((1u << lane) - 1))] = (unsigned char)lane;
+                constexpr int per_group = kEsUnits / kEsNW;
+                if (lane <= kEsNW)                             // where each plane group's units start
+                    s_off[slot][lane] = (unsigned char)__popcll(mask & ((1ull << (lane * per_group)) - 1));
+                if (lane == 0 && !mask) *(volatile int *)s_stop = k;
+            }
+        }
+        if (any_producer(late)) return EsOpen::leave;
+        if (*(volatile int *)s_stop != k) return EsOpen::copy;
+        tc::mbar_arrive(&full[st]);
+        if (tid == 0) tc::mbar_arrive(&full[st]);
+        return EsOpen::done;
+    }
+    __device__ __forceinline__ void copy(int k, int s, int st)
+    {
+        // a producer warp copies whole planes: 16 lanes a row, two rows a step
+        const int tid = threadIdx.x - 32 * kEsWarps, lane = tid & 31, ch = lane & 15, row0 = lane >> 4;
+        const long su = axis ? (long)a.gpx * a.wy : a.gpx, sw = axis ? a.gpx : (long)a.gpx * a.wy;
+        const int nw = axis ? a.wy : a.wz, Q = a.geo.Q, gw0 = W0 + h.ow + 4 * s;
+        for (int pl = tid >> 5; pl < 4 && gw0 + pl < nw; pl += kEsProducers / 32)
+            for (int c = ch; c < cols; c += 16) {
+                const float *src = src0 + (gw0 + pl) * sw + (gu0 + row0) * su + 4 * c;
+                uint32_t dst = ring0 + st * stage_bytes + 4u * (uint32_t)(pl * Q + row0 * P + 4 * c);
+#pragma unroll 4
+                for (int row = row0; row < rows; row += 2) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+                    src += 2 * su;
+                    dst += 8 * P;
+                }
+            }
+        copies_arrive(&full[st]);
+        if (tid == 0) tc::mbar_arrive(&full[st]);              // publishes the list
+    }
+};
+
 template <int P> __global__ void __launch_bounds__(kEsThreads, 1) erode_stream_kernel(EsArgs a, EsTiles t)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -247,69 +337,9 @@ template <int P> __global__ void __launch_bounds__(kEsThreads, 1) erode_stream_k
         if (v > 0.f) s_live[i / (32 * kEsX)] = 1;
     }
     __syncthreads();
-    int st = 0;
-    uint32_t ph = 0;
     if (warp >= kEsWarps) {
-        // producers: copy the planes of every orientation of this kind into the ring
-        const int tid = threadIdx.x - 32 * kEsWarps;
-        const long su = axis ? (long)a.gpx * a.wy : a.gpx, sw = axis ? a.gpx : (long)a.gpx * a.wy;
-        const int nu = axis ? a.wz : a.wy, nw = axis ? a.wy : a.wz;
-        bool wrapped = false;
-        for (int k = 0; k < k1 - k0; ++k) {
-            const int ob = s_ob[k], slot = k % kEsSlots;
-            const EsOrient h = a.head[a.orient_base + ob];
-            // a producer warp copies whole planes: 16 lanes a row, two rows a step
-            const int ch = lane & 15, row0 = lane >> 4;
-            const int cols = min(h.quads, (a.gpx - (X0 + h.ox)) >> 2);   // columns the window's rows have from here
-            const int gu0 = U0 + h.ou, rows = min(h.rows, nu - gu0);
-            const float *src0 = a.g + ob * a.g_so + X0 + h.ox;
-            bool stop = false;
-            for (int s = 0; s < kEsNW + h.lists; ++s) {
-                if (wrapped && !tc::mbar_wait(&empty[st], ph ^ 1)) {
-                    // a stage was not given back in time: wait for this thread's own copies and leave
-                    if (a.status) atomicCAS(a.status, 0, (int)IMF_ERR_TIMEOUT);
-                    asm volatile("cp.async.wait_all;\n" ::: "memory");
-                    return;
-                }
-                if (s == 0) {
-                    // the orientation's descriptors; the slot's last readers, four orientations back, gave
-                    // back their stages at least ten stages ago (an orientation has three or more)
-                    for (int i = tid; i < h.words / 4; i += kEsProducers)
-                        reinterpret_cast<int4 *>(s_words + slot * a.geo.words)[i] = __ldg(reinterpret_cast<const int4 *>(a.words + h.word0) + i);
-                    // the units that still have work, as one warp sees them; none: the block is done
-                    if (tid < 32) {
-                        const uint32_t mask = __ballot_sync(0xffffffffu, ((volatile unsigned char *)s_live)[lane] != 0);
-                        if (mask >> lane & 1) s_list[slot][__popc(mask & ((1u << lane) - 1))] = (unsigned char)lane;
-                        constexpr int per_group = kEsUnits / kEsNW;
-                        if (lane <= kEsNW)                     // where each plane group's units start
-                            s_off[slot][lane] = (unsigned char)__popcll(mask & ((1ull << (lane * per_group)) - 1));
-                        if (lane == 0 && !mask) *(volatile int *)&s_stop = k;
-                    }
-                    asm volatile("bar.sync 1, %0;\n" ::"n"(kEsProducers) : "memory");
-                    stop = *(volatile int *)&s_stop == k;
-                }
-                if (stop) {
-                    tc::mbar_arrive(&full[st]);
-                    if (tid == 0) tc::mbar_arrive(&full[st]);
-                    return;
-                }
-                const int gw0 = W0 + h.ow + 4 * s;
-                for (int pl = tid >> 5; pl < 4 && gw0 + pl < nw; pl += kEsProducers / 32)
-                    for (int c = ch; c < cols; c += 16) {
-                        const float *src = src0 + (gw0 + pl) * sw + (gu0 + row0) * su + 4 * c;
-                        uint32_t dst = ring0 + st * stage_bytes + 4u * (uint32_t)(pl * Q + row0 * P + 4 * c);
-#pragma unroll 4
-                        for (int row = row0; row < rows; row += 2) {
-                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-                            src += 2 * su;
-                            dst += 8 * P;
-                        }
-                    }
-                copies_arrive(&full[st]);
-                if (tid == 0) tc::mbar_arrive(&full[st]);      // publishes the list
-                if (++st == NS) { st = 0; ph ^= 1; wrapped = true; }
-            }
-        }
+        EsProducer<P> io{a, s_ob, s_words, s_live, s_list, s_off, full, empty, &s_stop, ring0, stage_bytes, axis, X0, U0, W0};
+        es_produce(io, k1 - k0, NS);
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         return;
     }
@@ -318,6 +348,8 @@ template <int P> __global__ void __launch_bounds__(kEsThreads, 1) erode_stream_k
     ring.base = smraw;
     ring.len = NS * stage_bytes;
     const uint32_t own = 4u * (uint32_t)((lane >> 3) * Q + (lane & 7));
+    int st = 0;
+    uint32_t ph = 0;
     int turn = warp;                                           // tasks until this warp's next one
     bool ok = true;
     for (int k = 0; k < k1 - k0 && ok; ++k) {

@@ -44,6 +44,36 @@ struct EsOrient {
     int word0, words;                // descriptor words, multiples of 4
 };
 
+// What a producer's orientation begins with, the same for every producer.
+enum class EsOpen { copy, done, leave };
+
+// Control flow of one producer thread over its `orientations` and the ring's `stages`. Io: steps(k), the stages of
+// orientation k; wait(st, phase), bounded, false when stage st was not given back in time; open(k, st, late), the
+// barrier that every producer of the block passes once an orientation, which is where they learn together that one
+// of them is late (leave) or that no output has work left (done); copy(k, s, st). A late thread copies nothing
+// more but goes on to that barrier: it counts all of them, and one that had left would hold the others there
+// without limit.
+template <class Io> __host__ __device__ __forceinline__ EsOpen es_produce(Io &io, int orientations, int stages)
+{
+    int st = 0;
+    uint32_t ph = 0;
+    bool wrapped = false, late = false;
+    for (int k = 0; k < orientations; ++k) {
+        const int steps = io.steps(k);
+        for (int s = 0; s < steps; ++s) {
+            if (wrapped && !late && !io.wait(st, ph ^ 1)) late = true;
+            if (s == 0) {
+                const EsOpen o = io.open(k, st, late);
+                if (o != EsOpen::copy) return o;
+            }
+            if (late) continue;
+            io.copy(k, s, st);
+            if (++st == stages) { st = 0; ph ^= 1; wrapped = true; }
+        }
+    }
+    return late ? EsOpen::leave : EsOpen::copy;
+}
+
 struct EsArgs {
     const float *g;
     long g_so;

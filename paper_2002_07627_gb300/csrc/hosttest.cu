@@ -1,8 +1,12 @@
 // Host-only exports that run the kernels' building blocks (fft.cuh, fft2.cuh, erode_plan.h,
 // fft_plan.h, orient_order.h, sweep_bits.cuh) on the CPU, for the CPU unit tests. Not part of
 // libimf and never loaded by the product path.
+#include <chrono>
 #include <cmath>
+#include <condition_variable>
 #include <cstring>
+#include <mutex>
+#include <thread>
 #include <vector>
 
 #include "fft.cuh"
@@ -189,4 +193,70 @@ extern "C" int imf_host_plan_sweep(const int *rk, int n_pts, const int *K, const
     if ((int)words.size() > max_words || h[0].words != (int)words.size()) return -2;
     std::memcpy(words_out, words.data(), words.size() * sizeof(int));
     return (int)words.size();
+}
+
+namespace {
+
+// The producers of one block of the streamed minimum on host threads: late[t * total + n] != 0 makes thread t's
+// wait for the n-th stage (over all orientations) run out.
+struct HostRing {
+    std::mutex m;
+    std::condition_variable cv;
+    int threads, arrived = 0, generation = 0;
+    bool any = false, result = false, stuck = false;
+
+    bool vote(bool late)
+    {
+        std::unique_lock<std::mutex> lock(m);
+        any = any || late;
+        const int mine = generation;
+        if (++arrived == threads) {
+            result = any;
+            any = false;
+            arrived = 0;
+            ++generation;
+            cv.notify_all();
+        } else if (!cv.wait_for(lock, std::chrono::seconds(2), [&] { return generation != mine || stuck; }) || stuck) {
+            stuck = true;                // some thread will never come: the device would wait for ever
+            cv.notify_all();
+            return true;
+        }
+        return result;
+    }
+};
+struct HostProducer {
+    HostRing &ring;
+    const int *n_steps;
+    const uint8_t *late;
+    int stop_at, n = 0, copied = 0;
+
+    int steps(int k) { return n_steps[k]; }
+    bool wait(int, uint32_t) { return !late[n]; }
+    imf::EsOpen open(int k, int, bool is_late)
+    {
+        if (ring.vote(is_late)) return imf::EsOpen::leave;
+        return k == stop_at ? imf::EsOpen::done : imf::EsOpen::copy;
+    }
+    void copy(int, int, int) { ++n; ++copied; }
+};
+
+} // namespace
+
+// Runs es_produce on `threads` host threads; how[t] gets 0 where thread t copied everything, 1 where it stopped at
+// orientation stop_at, 2 where it left on a timeout, and copied[t] its stages. Returns 1 when a thread was
+// left waiting at the producers' barrier, else 0.
+extern "C" int imf_host_stream_producers(int threads, int orientations, const int *n_steps, int stages, int stop_at,
+                                         const uint8_t *late, int total, int *how, int *copied)
+{
+    HostRing ring;
+    ring.threads = threads;
+    std::vector<std::thread> pool;
+    for (int t = 0; t < threads; ++t)
+        pool.emplace_back([&, t] {
+            HostProducer io{ring, n_steps, late + (size_t)t * total, stop_at};
+            how[t] = (int)imf::es_produce(io, orientations, stages);
+            copied[t] = io.copied;
+        });
+    for (auto &p : pool) p.join();
+    return ring.stuck;
 }

@@ -82,6 +82,48 @@ def test_stream_plan_refuses_cutters_too_wide_for_its_rows():
     assert _plan(wide, wide.max(0))[0] == -1
 
 
+def _producers(steps, stages, late, stop_at=-1):
+    from paper_2002_07627_gb300 import build
+    build.build()
+    L = ctypes.CDLL(build.HOSTLIB)
+    threads, total = late.shape
+    steps = np.asarray(steps, np.int32)
+    late = np.ascontiguousarray(late, np.uint8)
+    how, copied = np.full(threads, -1, np.int32), np.full(threads, -1, np.int32)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    stuck = L.imf_host_stream_producers(threads, len(steps), p(steps), stages, stop_at, p(late), total, p(how), p(copied))
+    return stuck, how.tolist(), copied.tolist()
+
+
+@pytest.mark.parametrize("stages", [3, 5, 10])
+@pytest.mark.parametrize("who", ["none", "first", "last", "all but one", "all", "at different stages"])
+def test_producers_leave_together_when_a_wait_runs_out(stages, who):
+    """The committed control flow of the producers on host threads, with waits that run out for some of them only:
+    nobody is left at the barrier they share, and whoever is not late leaves no later than the next orientation."""
+    steps = [4, 3, 6, 3, 5, 4]
+    total, threads = sum(steps), 6
+    for at in range(stages, total):
+        late = np.zeros((threads, total), np.uint8)
+        hit = {"none": [], "first": [0], "last": [threads - 1], "all but one": range(1, threads), "all": range(threads),
+               "at different stages": range(threads)}[who]
+        for t in hit:
+            late[t, min(at + (t if who == "at different stages" else 0), total - 1):] = 1
+        stuck, how, copied = _producers(steps, stages, late)
+        assert not stuck
+        ends = np.cumsum(steps)
+        first = min((int(np.argmax(late[t])) for t in hit), default=total)
+        nxt = int(ends[np.searchsorted(ends, first)]) if hit else total   # where its orientation ends
+        for t in range(threads):
+            own = int(np.argmax(late[t])) if late[t].any() else total
+            assert copied[t] == min(own, nxt)
+            assert how[t] == (0 if copied[t] == total else 2)
+
+
+def test_producers_stop_together_where_no_output_has_work_left():
+    stuck, how, copied = _producers([3, 4, 3], 3, np.zeros((4, 10), np.uint8), stop_at=1)
+    assert not stuck and how == [1] * 4 and copied == [3] * 4
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,r,n_orient", [((32, 24, 8), 3, 1900), ((33, 25, 9), 2, 200), ((70, 45, 37), 3, 40),
                                           ((31, 60, 17), 6, 90), ((5, 3, 2), 1, 930), ((97, 2, 30), 2, 160)])
