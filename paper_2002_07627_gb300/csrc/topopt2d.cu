@@ -559,7 +559,8 @@ imf_status imf_to2d_update(imf_to2d h, const float *xi, const float *S, const ui
         // they and S^eta stay inside the FP64 range for any float S
         imf_to::OcArgs a{};
         a.n = h->ne; a.xi = xi; a.S = S; a.passive = passive; a.volfrac = volfrac; a.move = move; a.eta = eta; a.beta = beta;
-        a.xs = h->s; a.out = xi_new; a.sc = h->sc; a.bar = h->bar;
+        a.xs = h->q;                     // free after an analysis; h->s is a sensitivity's, which may still be running
+        a.out = xi_new; a.sc = h->sc; a.bar = h->bar;
         TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
         TO_CU(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), s));
         TO_CU(imf_to::oc_solve(a, s));
