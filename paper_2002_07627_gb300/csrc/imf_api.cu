@@ -653,6 +653,23 @@ size_t work_bytes(imf_handle h, const WorkSizes &w, int slots)
     return t;
 }
 
+// The handle's small device words (dev_small). They are zero when this returns, not only once the default stream
+// gets there: the calls that use them run on the caller's streams, which need not be ordered with it.
+imf_status ensure_small(imf_handle h)
+{
+    if (h->dev_small) return IMF_OK;
+    int *p = nullptr;
+    TRY(dalloc(h, &p, (size_t)8));
+    cudaError_t e = cudaMemsetAsync(p, 0, 8 * sizeof(int), cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+        dfree(h, p);
+        return fail(h, IMF_ERR_CUDA, "clearing the small words: %s", cudaGetErrorString(e));
+    }
+    h->dev_small = p;
+    return IMF_OK;
+}
+
 imf_status ensure_work(imf_handle h)
 {
     const imf_options &op = h->opt;
@@ -665,8 +682,7 @@ imf_status ensure_work(imf_handle h)
         TRY(dalloc(h, &h->f, (size_t)N));
         h->awords = (op.nx + 31) / 32;
         TRY(dalloc(h, &h->A, (size_t)op.nz * op.ny * h->awords));
-        TRY(dalloc(h, &h->dev_small, (size_t)8));
-        CU(cudaMemset(h->dev_small, 0, 8 * sizeof(int)));
+        TRY(ensure_small(h));
     }
     if (rs > h->rho_spec_n) { dfree(h, h->rho_spec, h->rho_spec_n); TRY(dalloc(h, &h->rho_spec, rs)); h->rho_spec_n = rs; }
     if (x1 > h->X1_n) { dfree(h, h->X1, h->X1_n); TRY(dalloc(h, &h->X1, x1)); h->X1_n = x1; }
@@ -1580,10 +1596,7 @@ imf_status imf_penalize_sensitivity(imf_handle h, float *sens, const float *rho_
     if (!(w_acc >= 0.0 && w_acc < 1.0)) return fail(h, IMF_ERR_INVALID_ARG, "w_acc %g outside [0, 1)", w_acc);
     const long N = (long)h->opt.nx * h->opt.ny * h->opt.nz;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    if (!h->dev_small) {
-        TRY(dalloc(h, &h->dev_small, (size_t)8));
-        CU(cudaMemset(h->dev_small, 0, 8 * sizeof(int)));
-    }
+    TRY(ensure_small(h));
     unsigned *mb = (unsigned *)(h->dev_small + 3);
     h->last_stream = s;
     h->used_stream = true;
