@@ -47,8 +47,19 @@ struct GridBarrier {
     }
 };
 
+// Calls launch(blocks) with `want` blocks, or half as many, and so on down to one, until they fit. What fits is not known
+// beforehand: a stream may own only some of the device's SMs (a green context).
+template <typename F> cudaError_t launch_fitting(long want, F &&launch)
+{
+    for (long n = std::max(1L, want);; n = (n + 1) / 2) {
+        const cudaError_t e = launch(n);
+        if (e != cudaErrorCooperativeLaunchTooLarge || n == 1) return e;
+        cudaGetLastError();              // the refused launch left it behind
+    }
+}
+
 // Launches kernel(args) cooperatively with `threads` threads a block and `want` blocks, or as many as the
-// device holds at once (the kernel's loops stride over the grid).
+// device holds at once, or fewer (launch_fitting; the kernel's loops stride over the grid).
 template <typename A> cudaError_t launch_cooperative(void (*kernel)(A), const A &args, int threads, long want, cudaStream_t s)
 {
     int dev = 0, sms = 0, per = 0;
@@ -58,8 +69,9 @@ template <typename A> cudaError_t launch_cooperative(void (*kernel)(A), const A 
     if (e != cudaSuccess) return e;
     const long most = (long)std::max(per, 1) * sms;
     void *p[1] = {const_cast<A *>(&args)};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kernel), dim3((unsigned)std::max(1L, std::min(most, want))),
-                                       dim3(threads), p, 0, s);
+    return launch_fitting(std::min(most, want), [&](long n) {
+        return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kernel), dim3((unsigned)n), dim3(threads), p, 0, s);
+    });
 }
 
 } // namespace imf

@@ -14,6 +14,7 @@
 #include "erode_plan.h"
 #include "erode_stream.h"
 #include "fft_plan.h"
+#include "grid_barrier.cuh"
 #include "orient_order.h"
 #include "sweep_bits.cuh"
 #include "sweep_plan.h"
@@ -259,4 +260,19 @@ extern "C" int imf_host_stream_producers(int threads, int orientations, const in
         });
     for (auto &p : pool) p.join();
     return ring.stuck;
+}
+
+// The choice of a cooperative launch's blocks (grid_barrier.cuh) against a launcher with room for `room` blocks that
+// otherwise returns `error`. Returns the blocks launched, or minus the error; tries gets the calls made.
+extern "C" int imf_host_launch_fitting(long want, long room, int error, int *tries)
+{
+    long got = 0;
+    *tries = 0;
+    const cudaError_t e = imf::launch_fitting(want, [&](long n) {
+        ++*tries;
+        if (n > room) return cudaErrorCooperativeLaunchTooLarge;
+        got = n;
+        return (cudaError_t)error;
+    });
+    return e == cudaSuccess ? (int)got : -(int)e;
 }

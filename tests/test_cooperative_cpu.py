@@ -1,0 +1,20 @@
+"""How many blocks a cooperative kernel gets where the stream owns fewer SMs than the device has."""
+import ctypes
+
+import pytest
+
+TOO_LARGE = 720      # cudaErrorCooperativeLaunchTooLarge
+
+
+@pytest.mark.parametrize("want,room", [(1216, 1216), (1216, 64), (1216, 63), (5, 4), (3, 1), (1, 1), (0, 1), (257, 16)])
+def test_a_launch_that_does_not_fit_is_made_with_fewer_blocks(want, room):
+    from paper_2002_07627_gb300 import build
+    build.build()
+    L = ctypes.CDLL(build.HOSTLIB)
+    tries = ctypes.c_int()
+    n = L.imf_host_launch_fitting(ctypes.c_long(want), ctypes.c_long(room), 0, ctypes.byref(tries))
+    assert 1 <= n <= room and tries.value <= 12
+    assert n == max(want, 1) if want <= room else 2 * n > room or room == 1
+    # another error is the launch's result, at once; where not one block fits, so is this one
+    assert L.imf_host_launch_fitting(ctypes.c_long(1), ctypes.c_long(1), 9, ctypes.byref(tries)) == -9 and tries.value == 1
+    assert L.imf_host_launch_fitting(ctypes.c_long(want), ctypes.c_long(0), 0, ctypes.byref(tries)) == -TOO_LARGE
