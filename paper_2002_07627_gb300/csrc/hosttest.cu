@@ -18,6 +18,7 @@
 #include "orient_order.h"
 #include "sweep_bits.cuh"
 #include "sweep_plan.h"
+#include "topopt2d_mg.cuh"
 
 extern "C" int imf_host_fft(int L, int sign, const float *in, float *out)
 {
@@ -275,4 +276,13 @@ extern "C" int imf_host_launch_fitting(long want, long room, int error, int *tri
         return (cudaError_t)error;
     });
     return e == cudaSuccess ? (int)got : -(int)e;
+}
+
+// Whether the analysis takes the result of a multigrid solve that ended with `done` and this barrier error word.
+extern "C" int imf_host_mg_converged(double done, unsigned barrier_error)
+{
+    double sc[imf_to::kScN] = {0};
+    sc[imf_to::kScDone] = done;
+    const unsigned bar[2] = {12345u, barrier_error};
+    return imf_to::mg_converged(sc, bar);
 }

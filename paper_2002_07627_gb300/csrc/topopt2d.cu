@@ -33,6 +33,10 @@ constexpr int kMgMaxIter = 600;
 
 // scalar slots: rz[3], pq[2], rr[3], ff, vol, cnt, change
 enum { S_RZ = 0, S_PQ = 3, S_RR = 5, S_FF = 8, S_VOL = 9, S_CNT = 10, S_CHG = 11, S_N = 16 };
+// the cooperative kernels' scalars lie in the same slots; their barrier words follow, so that one memset clears
+// and one copy reads both
+constexpr size_t kScalarBytes = (S_N + 1) * sizeof(double);
+static_assert(imf_to::kScN == S_N && 2 * sizeof(unsigned) == sizeof(double), "scalars, then two barrier words");
 
 inline int blocks(long n, int cap = 152 * 8)
 {
@@ -331,10 +335,9 @@ struct imf_to2d_s {
     long ne = 0, ndof = 0;
     double *k0 = nullptr, *E = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr,
            *diag = nullptr, *sc = nullptr, *s = nullptr;
-    void *mem = nullptr;                 // what the pointers above and `bar` lie in
+    void *mem = nullptr;                 // what the pointers above lie in
     void *mg_mem = nullptr;              // multigrid hierarchy, behind them in `mem`, or NULL where it did not fit
     imf_to::MgArgs mg{};
-    unsigned *bar = nullptr;
     double compliance = 0.0, rel_res = 0.0;
     int iters = 0;
     bool have_u = false;
@@ -401,9 +404,8 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
     };
     const size_t v = h->ndof * sizeof(double), e = h->ne * sizeof(double);
     const Part parts[] = {{(void **)&h->k0, 64 * sizeof(double)}, {(void **)&h->E, e}, {(void **)&h->s, e},
-                          {(void **)&h->sc, S_N * sizeof(double)}, {(void **)&h->bar, 2 * sizeof(unsigned)},
-                          {(void **)&h->x, v}, {(void **)&h->r, v}, {(void **)&h->z, v}, {(void **)&h->p, v},
-                          {(void **)&h->q, v}, {(void **)&h->diag, v}};
+                          {(void **)&h->sc, kScalarBytes}, {(void **)&h->x, v}, {(void **)&h->r, v},
+                          {(void **)&h->z, v}, {(void **)&h->p, v}, {(void **)&h->q, v}, {(void **)&h->diag, v}};
     size_t total = 0;
     for (const Part &q : parts) total += (q.bytes + 255) / 256 * 256;
     // the multigrid hierarchy (about 530 bytes a node) follows them where it fits; without it the plain
@@ -436,7 +438,7 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
         h->mg.p1 = h->z;
         h->mg.q = h->q;
         h->mg.sc = h->sc;
-        h->mg.bar = h->bar;
+        h->mg.bar = reinterpret_cast<unsigned *>(h->sc + S_N);
     }
     *out = h;
     return IMF_OK;
@@ -474,15 +476,17 @@ imf_status imf_to2d_analyze(imf_to2d h, const float *rho, const double *force, c
         a.fixed = fixed;
         a.tol2 = o.cg_tol * o.cg_tol;
         a.max_iter = o.cg_max_iter < kMgMaxIter ? o.cg_max_iter : kMgMaxIter;
-        TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
-        TO_CU(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), s));
+        TO_CU(cudaMemsetAsync(h->sc, 0, kScalarBytes, s));
         imf_to::mg_setup(a, s);
         TO_CU(imf_to::mg_solve(a, s));
         if (u_out) TO_CU(cudaMemcpyAsync(u_out, h->x, h->ndof * sizeof(double), cudaMemcpyDeviceToDevice, s));
-        double res[imf_to::kScN];
+        double res[S_N + 1];
+        static_assert(sizeof res == kScalarBytes, "");
         TO_CU(cudaMemcpyAsync(res, h->sc, sizeof res, cudaMemcpyDeviceToHost, s));
         TO_CU(cudaStreamSynchronize(s));
-        if (res[imf_to::kScDone] == 1.0) {
+        unsigned bar[2];
+        std::memcpy(bar, res + S_N, sizeof bar);
+        if (imf_to::mg_converged(res, bar)) {
             h->compliance = res[imf_to::kScC];
             h->iters = (int)res[imf_to::kScIt];
             h->rel_res = res[imf_to::kScFf] > 0 ? std::sqrt(res[imf_to::kScLast] / res[imf_to::kScFf]) : 0.0;
@@ -560,15 +564,14 @@ imf_status imf_to2d_update(imf_to2d h, const float *xi, const float *S, const ui
         imf_to::OcArgs a{};
         a.n = h->ne; a.xi = xi; a.S = S; a.passive = passive; a.volfrac = volfrac; a.move = move; a.eta = eta; a.beta = beta;
         a.xs = h->q;                     // free after an analysis; h->s is a sensitivity's, which may still be running
-        a.out = xi_new; a.sc = h->sc; a.bar = h->bar;
-        TO_CU(cudaMemsetAsync(h->sc, 0, S_N * sizeof(double), s));
-        TO_CU(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), s));
+        a.out = xi_new; a.sc = h->sc; a.bar = reinterpret_cast<unsigned *>(h->sc + S_N);
+        TO_CU(cudaMemsetAsync(h->sc, 0, kScalarBytes, s));
         TO_CU(imf_to::oc_solve(a, s));
-        double r[9];
+        double r[S_N + 1];
         unsigned bar[2];
         TO_CU(cudaMemcpyAsync(r, h->sc, sizeof r, cudaMemcpyDeviceToHost, s));
-        TO_CU(cudaMemcpyAsync(bar, h->bar, sizeof bar, cudaMemcpyDeviceToHost, s));
         TO_CU(cudaStreamSynchronize(s));
+        std::memcpy(bar, r + S_N, sizeof bar);
         if (bar[1]) return fail(h, IMF_ERR_TIMEOUT, "optimality-criteria update: a grid barrier timed out");
         if (change_out) *change_out = r[6] > 0 ? r[7] / r[6] : 0.0;
         if (vol_out) *vol_out = r[6] > 0 ? r[8] / r[6] : 0.0;

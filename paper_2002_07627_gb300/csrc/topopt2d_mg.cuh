@@ -37,6 +37,9 @@ struct MgArgs {
     int max_iter;
 };
 enum { kScPq = 0, kScRr = 3, kScRz = 6, kScFf = 9, kScC = 10, kScIt = 11, kScDone = 12, kScLast = 13, kScN = 16 };
+// Whether a solve's scalars can be used: it converged and no block gave up at a barrier. A block that did has left
+// without its share of the compliance, while the others may still have passed that barrier and finished.
+inline bool mg_converged(const double *sc, const unsigned *bar) { return sc[kScDone] == 1.0 && bar[1] == 0; }
 
 // device bytes of the hierarchy's arrays; fills every level's sizes (0: too many levels)
 size_t mg_plan(int nx, int ny, double nu, MgArgs &a);

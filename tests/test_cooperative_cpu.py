@@ -18,3 +18,12 @@ def test_a_launch_that_does_not_fit_is_made_with_fewer_blocks(want, room):
     # another error is the launch's result, at once; where not one block fits, so is this one
     assert L.imf_host_launch_fitting(ctypes.c_long(1), ctypes.c_long(1), 9, ctypes.byref(tries)) == -9 and tries.value == 1
     assert L.imf_host_launch_fitting(ctypes.c_long(want), ctypes.c_long(0), 0, ctypes.byref(tries)) == -TOO_LARGE
+
+
+def test_a_solve_in_which_a_block_gave_up_is_not_taken():
+    """A block that gives up at the last barrier leaves without its share of the compliance, while the others pass
+    the barrier and report that the iteration converged."""
+    from paper_2002_07627_gb300 import build
+    build.build()
+    taken = lambda done, err: ctypes.CDLL(build.HOSTLIB).imf_host_mg_converged(ctypes.c_double(done), ctypes.c_uint(err))
+    assert taken(1.0, 0) == 1 and taken(1.0, 1) == 0 and taken(0.0, 0) == 0 and taken(0.0, 1) == 0
