@@ -1649,11 +1649,11 @@ imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, cons
     const long awords = (op.nx + 31) / 32;
     const long words = (long)op.nz * op.ny * awords;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    if ((size_t)words > h->plan_rem_n) {
+    if (2 * (size_t)words > h->plan_rem_n) {
         dfree(h, h->plan_rem);
         h->plan_rem_n = 0;
-        TRY(dalloc(h, &h->plan_rem, (size_t)words));
-        h->plan_rem_n = (size_t)words;
+        TRY(dalloc(h, &h->plan_rem, 2 * (size_t)words));
+        h->plan_rem_n = 2 * (size_t)words;
     }
     // counters (three sets in turn), barrier, results, removed voxels and order, in 8-byte words
     const size_t nc = 3 * ((size_t)n_sets + 1), need = nc + 1 + 3 + (size_t)n_sets + ((size_t)n_sets + 1) / 2;
@@ -1667,7 +1667,7 @@ imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, cons
     h->used_stream = true;
     {
         Launch L(h, KID_PLAN, s);
-        launch_plan_init(rho_omega, fixture, op.nx, op.ny, op.nz, (int)awords, op.tau, h->plan_rem, s);
+        launch_plan_init(rho_omega, fixture, op.nx, op.ny, op.nz, (int)awords, op.tau, h->plan_rem + words, s);
     }
     PlanArgs a{};
     a.sets = sets; a.words = words; a.n_sets = n_sets; a.max_steps = max_steps; a.rem = h->plan_rem;

@@ -182,7 +182,7 @@ struct PlanArgs {
     const uint32_t *sets;        // [n_sets][words]
     long words;
     int n_sets, max_steps;
-    uint32_t *rem;               // remaining negative space, cleared as the plan goes
+    uint32_t *rem;               // 2 x words; N in the second half, both overwritten as the plan goes
     unsigned long long *counts;  // 3 (n_sets + 1), zeroed by the caller
     unsigned *bar;               // grid barrier, two words, zeroed by the caller
     int *order;                  // min(max_steps, n_sets)

@@ -224,59 +224,89 @@ __global__ void plan_init_kernel(const float *rho, const uint8_t *fix, int nx, i
     }
 }
 
-// The whole greedy plan in one cooperative launch. A thread owns words of the negative space for good; per
-// step every block counts, for each set, the bits of its words that the set covers (shared counters, then one
-// atomic per set and block), and after a grid barrier each block finds the best set and clears its bits from
-// its own words. Words that are empty are not read again, so a step costs what is left of N. Bound by the
-// grid barrier and the latency of the first passes over the sets' words (in L2). Accessible sets and plan of
-// a 128^3 design with 64 sets, about 44 steps: 8.25 ms with three calls and a host round trip a step, 6.56 so
-// (0.5 of it from the minimum's streamed kernel).
-constexpr int kPlanChunk = 2048;         // sets counted at a time
+// The whole greedy plan in one cooperative launch. Blocks are units of (chunk of kPlanWords words, part of the
+// sets): a block lists the words of its chunk that still hold some of N and each of its warps counts, set by set, the
+// bits of them that the set covers; after a grid barrier every block finds the best set. So the sets of a small grid
+// spread over the SMs, and a step costs what is left of N. What is left lies in two buffers in turn: the parts of a
+// chunk all read the state before the last step and take that step's set out themselves, the first part writes
+// the result for the next step, and no second barrier is needed.
+// Bound by the grid barrier and the latency of the reads of the sets' words (in L2).
+// Random sets, ms for the whole plan (steps), with a host round trip a step, with words alone split over the
+// blocks (and sets one after another in each), and so: 128^3 x 64 sets (64) 2.67, 1.39, 0.81; 64^3 x 256 (116) 3.69,
+// 7.99, 0.95; 32^3 x 1024 (72) 2.34, 19.3, 0.54; 64 x 64 x 4096 (40) 1.59, 42.6, 0.37; 128^3 x 4096 (130) 189, 264, 60.6.
+constexpr int kPlanWords = 256;
 
-__global__ void __launch_bounds__(256) plan_greedy_kernel(const __grid_constant__ PlanArgs a)
+__host__ __device__ inline long plan_chunks(long words) { return (words + kPlanWords - 1) / kPlanWords; }
+
+__global__ void __launch_bounds__(kPlanWords) plan_greedy_kernel(const __grid_constant__ PlanArgs a)
 {
-    __shared__ unsigned cnt[kPlanChunk];
-    __shared__ unsigned long long best_key[8];
-    __shared__ int best_at[8];
+    constexpr int kWarps = kPlanWords / 32;
+    __shared__ uint32_t left[kPlanWords];
+    __shared__ int at[kPlanWords], found[kWarps];
+    __shared__ unsigned long long best_key[kWarps];
+    __shared__ int best_at[kWarps];
     GridBarrier g;
     g.bar = a.bar;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long step = (long)gridDim.x * 256, first = (long)blockIdx.x * 256 + threadIdx.x;
-    const int counters = a.n_sets + 1;       // the last one counts what is left of N itself
+    const int counters = a.n_sets + 1;       // the last one counts N itself (first pass)
+    const long chunks = plan_chunks(a.words);
+    // a part has at least a set for each warp
+    const long parts = max(1L, min((long)gridDim.x / chunks, ((long)a.n_sets + kWarps - 1) / kWarps));
+    const uint32_t *last = nullptr;          // the set of the step before
     int k = 0;
     unsigned long long total = 0, rest = 0;
     while (true) {
         unsigned long long *now = a.counts + (long)(k % 3) * counters;
-        for (int c0 = 0; c0 < counters; c0 += kPlanChunk) {
-            const int cn = min(kPlanChunk, counters - c0);
+        const uint32_t *src = a.rem + (k & 1 ? 0 : a.words);
+        uint32_t *dst = a.rem + (k & 1 ? a.words : 0);
+        for (long u = blockIdx.x; u < chunks * parts; u += gridDim.x) {
+            const long chunk = u % chunks, part = u / chunks, w = chunk * kPlanWords + threadIdx.x;
+            uint32_t v = w < a.words ? __ldcg(src + w) : 0u;
+            if (v && last) v &= ~__ldg(last + w);
+            if (part == 0 && w < a.words) __stcg(dst + w, v);
+            const unsigned some = __ballot_sync(0xffffffffu, v != 0);
+            __syncthreads();                 // the list of the unit before is read
+            if (lane == 0) found[warp] = __popc(some);
             __syncthreads();
-            for (int i = threadIdx.x; i < cn; i += 256) cnt[i] = 0;
-            __syncthreads();
-            for (long w = first - lane; w < a.words; w += step) {
-                const uint32_t rem = w + lane < a.words ? a.rem[w + lane] : 0u;
-                if (!__any_sync(0xffffffffu, rem != 0)) continue;
-                const uint32_t *s = a.sets + (long)c0 * a.words + w + lane;
-#pragma unroll 4
-                for (int i = 0; i < cn; ++i) {
-                    const uint32_t v = c0 + i == a.n_sets ? rem : rem ? rem & __ldg(s + (long)i * a.words) : 0u;
-                    const unsigned sum = __reduce_add_sync(0xffffffffu, (unsigned)__popc(v));
-                    if (lane == 0 && sum) atomicAdd(cnt + i, sum);
-                }
+            int n = 0, base = 0;
+#pragma unroll
+            for (int i = 0; i < kWarps; ++i) {
+                if (i == warp) base = n;
+                n += found[i];
+            }
+            if (v) {
+                const int i = base + __popc(some & ((1u << lane) - 1));
+                left[i] = v;
+                at[i] = (int)(w - chunk * kPlanWords);
             }
             __syncthreads();
-            for (int i = threadIdx.x; i < cn; i += 256)
-                if (cnt[i]) atomicAdd(now + c0 + i, (unsigned long long)cnt[i]);
+            if (!n) continue;
+            const int i1 = (int)((part + 1) * a.n_sets / parts);
+            for (int i = (int)(part * a.n_sets / parts) + warp; i < i1; i += kWarps) {
+                const uint32_t *set = a.sets + (long)i * a.words + chunk * kPlanWords;
+                unsigned c = 0;
+#pragma unroll 8
+                for (int j = lane; j < n; j += 32) c += __popc(left[j] & __ldg(set + at[j]));
+                c = __reduce_add_sync(0xffffffffu, c);
+                if (lane == 0 && c) atomicAdd(now + i, (unsigned long long)c);
+            }
+            if (k == 0 && part == 0 && warp == 0) {
+                unsigned c = 0;
+                for (int j = lane; j < n; j += 32) c += __popc(left[j]);
+                c = __reduce_add_sync(0xffffffffu, c);
+                if (lane == 0) atomicAdd(now + a.n_sets, (unsigned long long)c);
+            }
         }
         if (!g.wait()) return;
         if (k == 0) rest = total = __ldcg(now + a.n_sets);
         // the counters of the step before are free again: nobody reads them past the barrier above
         if (blockIdx.x == 0)
-            for (int i = threadIdx.x; i < counters; i += 256) a.counts[(long)((k + 2) % 3) * counters + i] = 0;
+            for (int i = threadIdx.x; i < counters; i += kPlanWords) a.counts[(long)((k + 2) % 3) * counters + i] = 0;
         if (k >= a.max_steps || rest == 0) break;
         // the set that covers the most, the lowest index among equals
         unsigned long long bk = 0;
         int bi = 0x7fffffff;
-        for (int i = threadIdx.x; i < a.n_sets; i += 256) {
+        for (int i = threadIdx.x; i < a.n_sets; i += kPlanWords) {
             const unsigned long long v = __ldcg(now + i);
             if (v > bk || (v == bk && i < bi)) { bk = v; bi = i; }
         }
@@ -290,23 +320,19 @@ __global__ void __launch_bounds__(256) plan_greedy_kernel(const __grid_constant_
         __syncthreads();
         bk = best_key[0];
         bi = best_at[0];
-        for (int i = 1; i < 8; ++i)
+        for (int i = 1; i < kWarps; ++i)
             if (best_key[i] > bk || (best_key[i] == bk && best_at[i] < bi)) { bk = best_key[i]; bi = best_at[i]; }
         if (bk == 0) break;
-        if (first == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
             a.order[k] = bi;
             a.removed[k] = (long long)bk;
         }
         rest -= bk;
         ++k;
-        const uint32_t *s = a.sets + (long)bi * a.words;
-        for (long w = first; w < a.words; w += step) {
-            const uint32_t rem = a.rem[w];
-            if (rem) a.rem[w] = rem & ~__ldg(s + w);
-        }
         if (rest == 0) break;
+        last = a.sets + (long)bi * a.words;
     }
-    if (first == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.result[0] = k;
         a.result[1] = (long long)total;
         a.result[2] = (long long)rest;
@@ -560,7 +586,7 @@ void launch_plan_init(const float *rho, const uint8_t *fix, int nx, int ny, int 
 
 cudaError_t launch_plan_greedy(const PlanArgs &a, cudaStream_t s)
 {
-    return launch_cooperative(plan_greedy_kernel, a, 256, (a.words + 255) / 256, s);
+    return launch_cooperative(plan_greedy_kernel, a, kPlanWords, plan_chunks(a.words) * ((a.n_sets + 7) / 8), s);
 }
 
 void launch_recheck_blocks(const RecheckArgs &a, int max_points, cudaStream_t s)

@@ -161,3 +161,25 @@ def test_normalisation_and_penalty_around_the_small_grid_limit(shape, fixture):
         ref = 0.7 * (s0 / m if m > 0 else s0) + 0.3 * s_imf
         assert np.abs(out - ref).max() <= 4e-7 * max(1.0, np.abs(ref).max())
     imf.close()
+
+
+@pytest.mark.parametrize("shape,n_sets,max_steps", [((1, 1, 8192), 9, None), ((1, 3, 8192), 8, None), ((4, 33, 70), 1025, 40),
+                                                    ((1, 16, 16), 5000, 12), ((30, 70, 4000), 3, None)])
+def test_greedy_plan_splits_words_and_sets_over_the_blocks(shape, n_sets, max_steps):
+    """One chunk of words and just over, parts of the sets that do not divide evenly, more sets than blocks and more
+    chunks than blocks: whole numbers, so equal to the oracle's."""
+    binding = _need()
+    import oracle
+    rng = np.random.default_rng(n_sets)
+    nz, ny, nx = shape
+    words = -(-nx // 32)
+    packed = rng.integers(0, 2**32, (n_sets, nz, ny, words), np.uint32)
+    for _ in range(3):
+        packed &= rng.integers(0, 2**32, packed.shape, np.uint32)
+    packed[n_sets // 3] = packed[n_sets - 1]
+    sets = [np.unpackbits(p.view(np.uint8), axis=-1, bitorder="little")[..., :nx].astype(bool) for p in packed]
+    rho = rng.uniform(0, 1, shape).astype(np.float32)
+    imf = binding.Imf(shape)
+    got = imf.process_plan(_dev(packed.view(np.int32)), _dev(rho), None, max_steps)
+    assert got == oracle.process_plan(sets, rho <= 0.5, max_steps)
+    imf.close()
