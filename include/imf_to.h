@@ -59,8 +59,8 @@ imf_status imf_to2d_project(imf_to2d h, const float *xi, float *rho, void *cuda_
  * [2 (nelx+1)(nely+1)] with the DEVICE uint8 dof mask `fixed` (nonzero = clamped, u = 0).
  * Keeps u in the handle (for imf_to2d_sensitivity) and copies it to `u_out` (DEVICE FP64, or
  * NULL). Synchronous. A conjugate gradient preconditioned by one multigrid V-cycle, in one launch;
- * where that does not reach cg_tol within 600 iterations (or its hierarchy, about 530 bytes a node, found
- * no memory), a Jacobi-preconditioned one from the start. Compliance, iteration count of the one that
+ * where that stalls (its residual does not halve for 400 iterations, or it reaches cg_max_iter; or its
+ * hierarchy, about 530 bytes a node, found no memory), a Jacobi-preconditioned one from the start. Compliance, iteration count of the one that
  * finished and relative residual via imf_to2d_result. Errors: IMF_ERR_INVALID_ARG,
  * IMF_ERR_CUDA; IMF_ERR_TIMEOUT when cg_max_iter is reached before cg_tol (u is the last
  * iterate). */

@@ -27,9 +27,15 @@ namespace {
 
 constexpr int kT = 256;
 constexpr int kCheckEvery = 16;      // CG iterations between residual checks on the host
-// multigrid-preconditioned iterations before the plain iteration takes over: designs of the loop take 40 to
-// 150 (256 x 128, contrast 1e3), and these cost what about 800 plain ones do
-constexpr int kMgMaxIter = 600;
+// When the plain iteration takes over from the multigrid-preconditioned one, whose iterations cost about two plain
+// ones (256 x 128: 50 against 24.8 us; 4 x 3: 12.6 against 19): once its residual has not halved for this many
+// iterations. Designs of the loop take 14 to 220 in all; checkerboards of 2 x 2 cells and random cells of contrast
+// 1e6 to 1e9 take 490 to 4000, falling in steps of up to 390 iterations, where the plain one takes 3300 to more
+// than 20000 (400 x 200 checkerboard, 1e6: 54 against 220 ms; a limit of 600 in all cost 264).
+constexpr int kMgPatience = 400;
+// On the coarsest grid alone the preconditioner is an inverse: 2 or 3 iterations, or it is one in name only (4 x 3
+// checkerboard of contrast 1e6: 1907 iterations against 48 plain ones).
+constexpr int kMgDirectIter = 4;
 
 // scalar slots: rz[3], pq[2], rr[3], ff, vol, cnt, change
 enum { S_RZ = 0, S_PQ = 3, S_RR = 5, S_FF = 8, S_VOL = 9, S_CNT = 10, S_CHG = 11, S_N = 16 };
@@ -475,7 +481,8 @@ imf_status imf_to2d_analyze(imf_to2d h, const float *rho, const double *force, c
         a.force = force;
         a.fixed = fixed;
         a.tol2 = o.cg_tol * o.cg_tol;
-        a.max_iter = o.cg_max_iter < kMgMaxIter ? o.cg_max_iter : kMgMaxIter;
+        a.max_iter = a.levels > 1 || o.cg_max_iter < kMgDirectIter ? o.cg_max_iter : kMgDirectIter;
+        a.patience = kMgPatience;
         TO_CU(cudaMemsetAsync(h->sc, 0, kScalarBytes, s));
         imf_to::mg_setup(a, s);
         TO_CU(imf_to::mg_solve(a, s));

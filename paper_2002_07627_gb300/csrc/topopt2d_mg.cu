@@ -523,7 +523,8 @@ __global__ void __launch_bounds__(T, 1) mg_solve_kernel(const __grid_constant__ 
     const double stop = a.tol2 * ff;
     bool done = ff == 0.0;
     double rr = ff, rz = 1.0, alpha = 0.0;
-    int it = 0;                              // iterations done
+    double best = ff;                        // |r|^2 that the last halving of |r| reached, and when
+    int it = 0, best_it = 0;                 // iterations done
     // Pass k applies iteration k's step to x and r (none in pass 0), then z = M^-1 r, then the next direction
     // and its product with the operator. r and p alternate between two buffers: neighbours read the old ones.
     while (!done) {
@@ -566,6 +567,14 @@ __global__ void __launch_bounds__(T, 1) mg_solve_kernel(const __grid_constant__ 
             rr = __ldcg(sc + kScRr + it % 3);
             done = rr <= stop;
             if (done || it >= a.max_iter) break;
+            if (it % 16 == 0) {
+                if (rr < 0.25 * best) {
+                    best = rr;
+                    best_it = it;
+                } else if (it - best_it >= a.patience) {
+                    break;                   // stalled: leave it to the plain iteration
+                }
+            }
         }
         // the sums of the pass before are free again: nobody reads them past the barrier above
         if (first == 0) {

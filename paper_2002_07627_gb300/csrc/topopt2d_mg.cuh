@@ -34,7 +34,7 @@ struct MgArgs {
     double *sc;                          // scalars, see kSc* (zeroed before the launch)
     unsigned *bar;                       // [0] barrier counter, [1] error (zeroed before the launch)
     double tol2;
-    int max_iter;
+    int max_iter, patience;              // most iterations, and most of them without the residual halving
 };
 enum { kScPq = 0, kScRr = 3, kScRz = 6, kScFf = 9, kScC = 10, kScIt = 11, kScDone = 12, kScLast = 13, kScN = 16 };
 // Whether a solve's scalars can be used: it converged and no block gave up at a barrier. A block that did has left
