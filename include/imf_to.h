@@ -60,7 +60,8 @@ imf_status imf_to2d_project(imf_to2d h, const float *xi, float *rho, void *cuda_
  * Keeps u in the handle (for imf_to2d_sensitivity) and copies it to `u_out` (DEVICE FP64, or
  * NULL). Synchronous. A conjugate gradient preconditioned by one multigrid V-cycle, in one launch;
  * where that stalls (its residual does not halve for 400 iterations, or it reaches cg_max_iter; or its
- * hierarchy, about 530 bytes a node, found no memory), a Jacobi-preconditioned one from the start. Compliance, iteration count of the one that
+ * hierarchy, about 530 bytes a node, found no memory or, above 256 MB, would have taken more than a
+ * sixteenth of what was free), a Jacobi-preconditioned one from the start. Compliance, iteration count of the one that
  * finished and relative residual via imf_to2d_result. Errors: IMF_ERR_INVALID_ARG,
  * IMF_ERR_CUDA; IMF_ERR_TIMEOUT when cg_max_iter is reached before cg_tol (u is the last
  * iterate). */

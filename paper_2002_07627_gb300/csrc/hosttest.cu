@@ -286,3 +286,9 @@ extern "C" int imf_host_mg_converged(double done, unsigned barrier_error)
     const unsigned bar[2] = {12345u, barrier_error};
     return imf_to::mg_converged(sc, bar);
 }
+
+// Whether an analysis handle takes a multigrid hierarchy of `bytes` where `room` bytes are free.
+extern "C" int imf_host_mg_affordable(unsigned long long bytes, unsigned long long room)
+{
+    return imf_to::mg_affordable((size_t)bytes, (size_t)room);
+}

@@ -414,9 +414,14 @@ imf_status imf_to2d_create(const imf_to2d_options *o, imf_to2d *out)
                           {(void **)&h->z, v}, {(void **)&h->p, v}, {(void **)&h->q, v}, {(void **)&h->diag, v}};
     size_t total = 0;
     for (const Part &q : parts) total += (q.bytes + 255) / 256 * 256;
-    // the multigrid hierarchy (about 530 bytes a node) follows them where it fits; without it the plain
-    // iteration does the work
-    const size_t mg_bytes = imf_to::mg_plan(o->nelx, o->nely, o->nu, h->mg);
+    // the multigrid hierarchy (about 530 bytes a node) follows them where it fits and leaves the device to others;
+    // without it the plain iteration does the work
+    size_t mg_bytes = imf_to::mg_plan(o->nelx, o->nely, o->nu, h->mg);
+    if (mg_bytes > imf_to::kMgFreeBytes) {
+        size_t room = 0, all = 0;
+        if (cudaMemGetInfo(&room, &all) != cudaSuccess) cudaGetLastError();
+        if (!imf_to::mg_affordable(mg_bytes, room > total ? room - total : 0)) mg_bytes = 0;
+    }
     if (mg_bytes && cudaMalloc(&h->mem, total + mg_bytes) == cudaSuccess) h->mg_mem = static_cast<char *>(h->mem) + total;
     else cudaGetLastError();
     if (!h->mg_mem && cudaMalloc(&h->mem, total) != cudaSuccess) {

@@ -41,6 +41,12 @@ enum { kScPq = 0, kScRr = 3, kScRz = 6, kScFf = 9, kScC = 10, kScIt = 11, kScDon
 // without its share of the compliance, while the others may still have passed that barrier and finished.
 inline bool mg_converged(const double *sc, const unsigned *bar) { return sc[kScDone] == 1.0 && bar[1] == 0; }
 
+// A hierarchy is five times what a handle holds without it. Above 256 MB (500,000 nodes) it is taken only where
+// it is at most a sixteenth of the device memory still free after the handle's own arrays, so that handles made later
+// find what they found before: on an empty device up to 33 million nodes (5800 x 5800).
+constexpr size_t kMgFreeBytes = (size_t)256 << 20;
+inline bool mg_affordable(size_t bytes, size_t room) { return bytes <= kMgFreeBytes || bytes <= room / 16; }
+
 // device bytes of the hierarchy's arrays; fills every level's sizes (0: too many levels)
 size_t mg_plan(int nx, int ny, double nu, MgArgs &a);
 // places the arrays of a planned hierarchy in `mem` (mg_plan bytes)

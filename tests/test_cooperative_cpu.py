@@ -27,3 +27,13 @@ def test_a_solve_in_which_a_block_gave_up_is_not_taken():
     build.build()
     taken = lambda done, err: ctypes.CDLL(build.HOSTLIB).imf_host_mg_converged(ctypes.c_double(done), ctypes.c_uint(err))
     assert taken(1.0, 0) == 1 and taken(1.0, 1) == 0 and taken(0.0, 0) == 0 and taken(0.0, 1) == 0
+
+
+def test_a_large_hierarchy_takes_a_sixteenth_of_the_free_memory_at_most():
+    from paper_2002_07627_gb300 import build
+    build.build()
+    L = ctypes.CDLL(build.HOSTLIB)
+    ok = lambda b, room: L.imf_host_mg_affordable(ctypes.c_ulonglong(b), ctypes.c_ulonglong(room))
+    G = 1 << 30
+    assert ok(256 << 20, 0) == 1 and ok((256 << 20) + 1, 4 * G) == 0 and ok((256 << 20) + 1, 5 * G) == 1
+    assert ok(16 * G, 256 * G) == 1 and ok(16 * G + 1, 256 * G) == 0 and ok(142 * G, 250 * G) == 0

@@ -38,3 +38,23 @@ def test_update_beside_a_running_sensitivity():
         torch.cuda.synchronize()
         assert torch.equal(sens, want_sens) and float((new - want_new).abs().max()) <= 1e-6
     to.close()
+
+
+def test_a_huge_grid_leaves_the_device_to_others():
+    """2^28 elements: the handle takes its own vectors (six of 2 doubles a node, two of a double an element), and the
+    multigrid hierarchy, five times that, is left out."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2002_07627_gb300 import binding, build
+    build.build()
+    torch.zeros(1, device="cuda")
+    n = 1 << 14
+    own = 6 * 16 * (n + 1) ** 2 + 2 * 8 * n * n
+    room = torch.cuda.mem_get_info()[0]
+    if room < own + (8 << 30):
+        pytest.skip("not enough free memory")
+    to = binding.To2d(n, n)
+    taken = room - torch.cuda.mem_get_info()[0]
+    to.close()
+    assert own <= taken <= own + room // 16
