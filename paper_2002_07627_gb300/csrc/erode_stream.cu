@@ -179,11 +179,6 @@ template <int X, int P> __device__ __forceinline__ void run_list(const int *d, c
     }
 }
 
-struct EsTiles {
-    int x, u[2], w[2];               // tiles along x, and along the run and plane axis of either kind
-    __host__ __device__ int kind(int a) const { return x * u[a] * w[a]; }
-};
-
 // the copies of this thread issued so far arrive on `bar` when they land
 __device__ __forceinline__ void copies_arrive(uint64_t *bar)
 {
@@ -403,16 +398,6 @@ template <int P> __global__ void __launch_bounds__(kEsThreads, 1) erode_stream_k
     }
 }
 
-EsTiles es_tile_counts(int nx, int ny, int nz)
-{
-    auto up = [](int n, int d) { return (n + d - 1) / d; };
-    EsTiles t{};
-    t.x = up(nx, kEsTX);
-    t.u[0] = up(ny, kEsRows); t.w[0] = up(nz, kEsW);
-    t.u[1] = up(nz, kEsRows); t.w[1] = up(ny, kEsW);
-    return t;
-}
-
 template <int P> bool launch_p(const EsArgs &a, const EsTiles &t, long blocks, cudaStream_t s)
 {
     const size_t smem = (size_t)a.geo.stages * 16 * a.geo.Q + kEsAccBytes + (size_t)kEsSlots * a.geo.words * 4;
@@ -425,12 +410,6 @@ template <int P> bool launch_p(const EsArgs &a, const EsTiles &t, long blocks, c
 }
 
 } // namespace
-
-long es_tiles(int nx, int ny, int nz)
-{
-    const EsTiles t = es_tile_counts(nx, ny, nz);
-    return (long)t.kind(0) + t.kind(1);
-}
 
 bool launch_erode_stream(const EsArgs &a, cudaStream_t s)
 {

@@ -34,6 +34,7 @@ __host__ __device__ constexpr int es_unroll(int L) { return L == 1 ? 4 : L <= 9 
 struct EsGeometry {
     int P = 0, R = 0, Q = 0, stages = 0;   // row pitch, rows per plane, plane pitch, stages of four planes
     int words = 0;                         // descriptor words of a slot (the most any orientation has)
+    double cost = 0;                       // shared loads of a thread per orientation, on average
 };
 
 struct EsOrient {
@@ -43,6 +44,21 @@ struct EsOrient {
     int ox, ou, ow;                  // tile origin = block output origin + (ox, ou, ow) in window index
     int word0, words;                // descriptor words, multiples of 4
 };
+
+// Output tiles of a grid: along x, and along the run and plane axis of either kind of orientation.
+struct EsTiles {
+    int x, u[2], w[2];
+    __host__ __device__ int kind(int a) const { return x * u[a] * w[a]; }
+};
+inline EsTiles es_tile_counts(int nx, int ny, int nz)
+{
+    auto up = [](int n, int d) { return (n + d - 1) / d; };
+    EsTiles t{};
+    t.x = up(nx, kEsTX);
+    t.u[0] = up(ny, kEsRows); t.w[0] = up(nz, kEsW);
+    t.u[1] = up(nz, kEsRows); t.w[1] = up(ny, kEsW);
+    return t;
+}
 
 // What a producer's orientation begins with, the same for every producer.
 enum class EsOpen { copy, done, leave };
@@ -89,7 +105,5 @@ struct EsArgs {
 };
 // false (nothing launched) where no instance applies
 bool launch_erode_stream(const EsArgs &a, cudaStream_t s);
-// output tiles of one orientation group (both run axes), for the choice of the groups
-long es_tiles(int nx, int ny, int nz);
 
 } // namespace imf

@@ -3,9 +3,11 @@
 // and the CPU tests (hosttest.cu).
 #pragma once
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <vector>
 
+#include "erode.cuh"
 #include "erode_stream.cuh"
 
 namespace imf {
@@ -52,7 +54,8 @@ inline bool es_plan(const std::vector<std::vector<int32_t>> &sh, const int K[3],
     std::vector<int> first(n + 1, 0), top(3 * (size_t)n, 0);
     head.assign(n, EsOrient{});
     words.clear();
-    int need = 0, eu = 0;
+    int need = 0, eu = 0, with_points = 0;
+    long loads = 0;
     std::vector<uint8_t> in;
     for (int o = 0; o < n; ++o) {
         EsOrient &h = head[o];
@@ -68,8 +71,11 @@ inline bool es_plan(const std::vector<std::vector<int32_t>> &sh, const int K[3],
         in.assign((size_t)e[0] * e[1] * e[2], 0);
         for (size_t m = 0; m < v.size(); m += 3)
             in[((size_t)(v[m + 2] - mn[2]) * e[1] + (v[m + 1] - mn[1])) * e[0] + (v[m] - mn[0])] = 1;
-        const int u = es_runs(in, e, mn, 1, nullptr) <= es_runs(in, e, mn, 2, nullptr) ? 1 : 2, w = 3 - u;
+        const long along_y = es_runs(in, e, mn, 1, nullptr), along_z = es_runs(in, e, mn, 2, nullptr);
+        const int u = along_y <= along_z ? 1 : 2, w = 3 - u;
         es_runs(in, e, mn, u, &runs);
+        loads += std::min(along_y, along_z);
+        ++with_points;
         first[o + 1] = (int)runs.size();
         for (int c = 0; c < 3; ++c) top[3 * o + c] = mx[c];
         const int shift = (K[0] - mx[0]) & 3;                  // copies start at multiples of 4 columns
@@ -83,6 +89,7 @@ inline bool es_plan(const std::vector<std::vector<int32_t>> &sh, const int K[3],
         need = std::max(need, 4 * h.quads);
         eu = std::max(eu, e[u] - 1);
     }
+    g.cost = (double)loads / std::max(with_points, 1);
     g.P = es_pitch(need);
     g.R = kEsRows + eu;
     g.Q = g.R * g.P;
@@ -123,6 +130,28 @@ inline bool es_plan(const std::vector<std::vector<int32_t>> &sh, const int K[3],
     if (slots > kEsBudget) return false;
     g.stages = (int)std::min<size_t>(kEsMaxStages, (kEsBudget - slots) / stage);
     return g.stages >= 3;
+}
+
+// Whether the streamed kernel takes a batch of nb orientations, kind[a] of them with runs along axis a, of a planned tool.
+// Its time over the tiled kernel's follows, to 11 % over 208 measurements (grids 40^3 to 128^3 and flat and
+// long ones, cutters of radius 1 to 11, 8 to 64 orientations),
+//   sqrt(V) (0.715 + (1.14 + 2.1 min(1, 300 / cost)) / p):
+// V is the volume of its tiles with their orientations over that of the tiled kernel's, p the pairs of a tile and an
+// orientation an SM gets, cost the loads of a thread per orientation. Its blocks fill a ring before they reduce, which
+// few pairs or cheap cutters do not pay for, and its tiles of 24 rows along z waste a flat grid. With the line at
+// twelve tiles x orientations of either kind an SM alone (us, tiled and streamed): 200 x 100 x 8 x 16, radius 1, 40 and 64;
+// 400 x 60 x 32 x 8, radius 1, 78 and 98; 200 x 100 x 8 x 32, radius 8, 690 and 766; 40^3 x 64, radius 2, 92 and 109.
+// Chosen by this, at most 1.07 (558 and 597) in those measurements. Grids of one plane use an eighth of its
+// tiles and stay with the tiled kernel.
+inline bool es_faster(const EsGeometry &g, int nx, int ny, int nz, const int kind[2], int nb, int nsm)
+{
+    const EsTiles t = es_tile_counts(nx, ny, nz);
+    const double pairs = (double)t.kind(0) * kind[0] + (double)t.kind(1) * kind[1];
+    if (nz < 2 || !(pairs > 0) || (double)(t.kind(0) + t.kind(1)) * nb < 12.0 * nsm) return false;
+    auto up = [](int n, int d) { return (double)((n + d - 1) / d); };
+    const double tiled = up(nx, kErTX) * up(ny, kErTY) * up(nz, kErTZ) * nb;
+    const double V = pairs * (kEsTX * kEsRows * kEsW) / (tiled * (kErTX * kErTY * kErTZ));
+    return std::sqrt(V) * (0.715 + (1.14 + 2.1 * std::min(1.0, 300.0 / std::max(g.cost, 1.0))) * nsm / pairs) < 1.0;
 }
 
 } // namespace imf

@@ -292,3 +292,22 @@ extern "C" int imf_host_mg_affordable(unsigned long long bytes, unsigned long lo
 {
     return imf_to::mg_affordable((size_t)bytes, (size_t)room);
 }
+
+// Whether a batch takes the streamed minimum (erode_stream.h): the sharp offsets of its orientations one after another,
+// count[o] of them each. cost gets the plan's loads of a thread per orientation, kind the orientations with runs along
+// y and along z. Returns -1 where the plan refuses the points.
+extern "C" int imf_host_stream_faster(const int *sh, const int *count, int n_orient, const int *K, int nx, int ny, int nz,
+                                      int nsm, double *cost, int *kind)
+{
+    std::vector<std::vector<int32_t>> v;
+    for (int o = 0; o < n_orient; sh += 3 * (size_t)count[o], ++o) v.emplace_back(sh, sh + 3 * (size_t)count[o]);
+    std::vector<imf::EsOrient> h;
+    std::vector<int> words;
+    imf::EsGeometry g;
+    if (!imf::es_plan(v, K, g, h, words)) return -1;
+    kind[0] = kind[1] = 0;
+    for (const imf::EsOrient &e : h)
+        if (e.axis >= 0) ++kind[e.axis];
+    *cost = g.cost;
+    return imf::es_faster(g, nx, ny, nz, kind, n_orient, nsm);
+}

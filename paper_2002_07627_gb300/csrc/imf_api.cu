@@ -1341,21 +1341,20 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         if (h->opt.sweep_loop && !h->aset) launch_sweep_loop(a, h->nsm, s);
         else launch_sweep(a, s);
     }
-    // The streamed kernel from about twelve (tile, orientation) pairs an SM on: below that its blocks are
-    // mostly ring fill. Measured with the tiled one (us, tiles x orientations): 48^3 98 against 87 (1152),
-    // 60x40x90 175 against 174 (1760), 40^3 199 against 215 (1920), 72^3 166 against 197 (2592), 80^3 438
-    // against 582 (11520). Grids of one plane use an eighth of its tiles and stay with the tiled kernel.
     bool streamed = false;
-    const long es_t = es_tiles(op.nx, op.ny, op.nz);
-    if (t.es_ok && op.erode_xt == 0 && !t.erode_levels && op.nz > 1 && es_t * nb >= 12L * h->nsm) {
+    int kind[2] = {0, 0};                // orientations of the batch with runs along y, along z
+    if (t.es_ok)
+        for (int i = o0; i < o0 + nb; ++i)
+            if (t.es_axis[i] >= 0) kind[(int)t.es_axis[i]]++;
+    if (t.es_ok && op.erode_xt == 0 && !t.erode_levels && es_faster(t.es, op.nx, op.ny, op.nz, kind, nb, h->nsm)) {
         EsArgs a{};
         a.g = h->g; a.g_so = gso; a.gpx = t.gpx; a.wx = t.win[0]; a.wy = t.win[1]; a.wz = t.win[2];
         a.head = t.es_head; a.words = t.es_words;
         a.nx = op.nx; a.ny = op.ny; a.nz = op.nz; a.orient_base = o0; a.nb = nb;
+        a.kind[0] = kind[0]; a.kind[1] = kind[1];
         a.f = h->f; a.status = h->dev_small; a.geo = t.es;
-        for (int i = o0; i < o0 + nb; ++i)
-            if (t.es_axis[i] >= 0) a.kind[t.es_axis[i]]++;
-        const long tiles = es_t;
+        const EsTiles et = es_tile_counts(op.nx, op.ny, op.nz);
+        const long tiles = (long)et.kind(0) + et.kind(1);
         // blocks per tile: about six waves of them (a block loads its outputs and fills its ring before
         // it reduces anything, so fewer and longer blocks win where the tiles alone fill the SMs), and
         // not below one and a half orientations each. Measured, ms: 256^3 x 64 a launch, 5632 tiles: 17.1

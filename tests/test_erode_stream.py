@@ -177,3 +177,64 @@ def test_planar_blocks_equal_the_3d_ones(n, cut, groups):
         got.append(raw.clone())
         imf.close()
     assert torch.equal(*got)
+
+
+def _choice(n, tool, nsm=152):
+    """(streamed or not, loads of a thread per orientation, orientations with runs along y / z) for one batch of all
+    the tool's orientations on an n = (nx, ny, nz) grid, from the plan that the library makes."""
+    from paper_2002_07627_gb300 import binding, build
+    build.build()
+    imf = binding.Imf(n[::-1], plan_only=True, precision=binding.IMF_FP32_FFT)
+    imf.set_tool(0, tool.holder, tool.cutter, tool.origin, tool.quats)
+    info = imf.tool_info(0)
+    sh = [imf.offsets(0, o, 2) for o in range(info.n_orient)]
+    imf.close()
+    count = np.array([len(v) for v in sh], np.int32)
+    flat = np.ascontiguousarray(np.concatenate(sh), np.int32)
+    K, cost, kind = np.array(info.kmax, np.int32), ctypes.c_double(), np.zeros(2, np.int32)
+    L = ctypes.CDLL(build.HOSTLIB)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    got = L.imf_host_stream_faster(p(flat), p(count), len(count), p(K), *n, nsm, ctypes.byref(cost), p(kind))
+    return got, cost.value, kind.tolist()
+
+
+@pytest.mark.parametrize("n,r,l,n_orient,want", [
+    ((200, 100, 8), 1, 1, 16, 0), ((200, 100, 8), 8, 20, 32, 0), ((400, 60, 32), 1, 3, 8, 0), ((40, 40, 40), 2, 5, 64, 0),
+    ((60, 40, 90), 2, 5, 32, 0), ((48, 48, 48), 3, 20, 24, 0), ((64, 64, 1), 3, 20, 64, 0), ((128, 128, 128), 3, 20, 64, 1),
+    ((96, 96, 96), 3, 20, 32, 1), ((75, 61, 50), 3, 20, 24, 1), ((128, 128, 128), 1, 1, 32, 1), ((40, 40, 40), 8, 20, 64, 1)])
+def test_the_streamed_minimum_is_taken_where_it_measured_faster(n, r, l, n_orient, want):
+    got, cost, kind = _choice(n, synth.cylinder_tool(r, l, r + 3, 8, synth.fibonacci_quats(n_orient)))
+    assert got == want and cost > 8 and sum(kind) == n_orient
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,r,l,n_orient", [((31, 60, 17), 6, 9, 120), ((40, 48, 40), 11, 3, 64), ((70, 45, 37), 3, 20, 64),
+                                            ((97, 2, 30), 4, 9, 160), ((5, 3, 2), 4, 9, 930), ((33, 49, 17), 4, 9, 300),
+                                            ((32, 24, 8), 3, 9, 1900)])
+@pytest.mark.parametrize("groups", [0, 1, 7])
+def test_streamed_minimum_equals_the_tiled_one_where_it_runs(n, r, l, n_orient, groups):
+    """As above, on cases that the rule does give to the streamed kernel (long runs, the widest pitch and the fewest
+    stages among them); a group that holds more orientations of a kind than a block can goes to the tiled kernel."""
+    torch = pytest.importorskip("torch")
+    from paper_2002_07627_gb300 import binding, build
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    quats = np.random.default_rng(n_orient).normal(size=(n_orient, 4))
+    tool = synth.cylinder_tool(r, l, r + 2, 4, quats)
+    chosen, _, kind = _choice(n, tool, torch.cuda.get_device_properties(0).multi_processor_count)
+    assert chosen == 1
+    assert groups != 1 or (max(kind) > 256) == (n_orient > 512)
+    rho = torch.from_numpy(synth.beam_density(n, n_beams=5, seed=3)).cuda()
+    got = []
+    for xt in (8, 0):
+        imf = binding.Imf(tuple(rho.shape), erode_xt=xt, erode_groups=groups, orient_batch=n_orient,
+                          precision=binding.IMF_FP32_FFT)
+        imf.set_tool(0, tool.holder, tool.cutter, tool.origin, tool.quats)
+        raw = torch.empty_like(rho)
+        fbar, sec = imf.compute(rho, raw=raw)
+        imf.sync()
+        got.append((raw.clone(), fbar.clone(), sec.clone()))
+        imf.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
