@@ -311,3 +311,21 @@ extern "C" int imf_host_stream_faster(const int *sh, const int *count, int n_ori
     *cost = g.cost;
     return imf::es_faster(g, nx, ny, nz, kind, n_orient, nsm);
 }
+
+// Whether a batch takes the sweep on staged tiles (sweep_plan.h): the cutter offsets of its orientations one after
+// another, count[o] of them each. runs gets the plan's runs along x. Returns -1 where the plan refuses the cutter.
+extern "C" int imf_host_sweep_faster(const int *rk, const int *count, int n_orient, const int *K, const int *kmin, int nx, int ny,
+                                     int nz, int nsm, double *runs)
+{
+    std::vector<std::vector<int32_t>> v;
+    for (int o = 0; o < n_orient; rk += 3 * (size_t)count[o], ++o) v.emplace_back(rk, rk + 3 * (size_t)count[o]);
+    std::vector<imf::SwOrient> h;
+    std::vector<int> words;
+    imf::SwGeometry g;
+    if (!imf::sw_plan(v, K, kmin, nx, g, h, words)) return -1;
+    int kind[2] = {0, 0};
+    for (const imf::SwOrient &e : h)
+        if (e.axis >= 0) ++kind[e.axis];
+    *runs = g.runs;
+    return imf::sw_faster(g, nx, ny, nz, kind, n_orient, nsm);
+}

@@ -83,6 +83,7 @@ struct Tool {
     int4 *sw_pairs = nullptr;            // sweep run descriptors (SweepArgs::pairs), all orientations
     int *sw_start = nullptr;
     bool sw_ok = false;                  // planned for the sweep on staged tiles (sweep_tile.cu)
+    std::vector<signed char> sw_axis;    // its run axis of every orientation
     SwGeometry sw;
     SwOrient *sw_head = nullptr;
     int *sw_words = nullptr;
@@ -1187,6 +1188,8 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
     std::vector<int> sw_words;
     t.sw_ok = sw_plan(t.rk, t.kmax, t.kmin, h->opt.nx, t.sw, sw_head, sw_words);
     if (!t.sw_ok) { sw_head.clear(); sw_words.clear(); }
+    t.sw_axis.clear();
+    for (const SwOrient &e : sw_head) t.sw_axis.push_back((signed char)e.axis);
     if (!plan_only) {
         int dev = 0, n = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
@@ -1302,7 +1305,13 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         Launch L(h, KID_RECHECK, s);
         launch_recheck_blocks(a, 152 * 64, s);     // up to 64 points (warps) in flight per SM
     }
-    if (h->run_sweep && t.sw_ok && !op.sweep_loop) {
+    // orientations of the batch by run axis, in the plan of the staged sweep and of the streamed minimum
+    int sw_kind[2] = {0, 0}, es_kind[2] = {0, 0};
+    for (int i = o0; i < o0 + nb; ++i) {
+        if (t.sw_ok && t.sw_axis[i] >= 0) sw_kind[(int)t.sw_axis[i]]++;
+        if (t.es_ok && t.es_axis[i] >= 0) es_kind[(int)t.es_axis[i]]++;
+    }
+    if (h->run_sweep && t.sw_ok && !op.sweep_loop && sw_faster(t.sw, op.nx, op.ny, op.nz, sw_kind, nb, h->nsm)) {
         SwArgs a{};
         a.bits = h->bits; a.b_so = bso; a.wpr = t.wpr; a.wy = t.win[1]; a.wz = t.win[2];
         a.head = t.sw_head; a.words = t.sw_words; a.nx = op.nx; a.ny = op.ny; a.nz = op.nz;
@@ -1342,16 +1351,12 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         else launch_sweep(a, s);
     }
     bool streamed = false;
-    int kind[2] = {0, 0};                // orientations of the batch with runs along y, along z
-    if (t.es_ok)
-        for (int i = o0; i < o0 + nb; ++i)
-            if (t.es_axis[i] >= 0) kind[(int)t.es_axis[i]]++;
-    if (t.es_ok && op.erode_xt == 0 && !t.erode_levels && es_faster(t.es, op.nx, op.ny, op.nz, kind, nb, h->nsm)) {
+    if (t.es_ok && op.erode_xt == 0 && !t.erode_levels && es_faster(t.es, op.nx, op.ny, op.nz, es_kind, nb, h->nsm)) {
         EsArgs a{};
         a.g = h->g; a.g_so = gso; a.gpx = t.gpx; a.wx = t.win[0]; a.wy = t.win[1]; a.wz = t.win[2];
         a.head = t.es_head; a.words = t.es_words;
         a.nx = op.nx; a.ny = op.ny; a.nz = op.nz; a.orient_base = o0; a.nb = nb;
-        a.kind[0] = kind[0]; a.kind[1] = kind[1];
+        a.kind[0] = es_kind[0]; a.kind[1] = es_kind[1];
         a.f = h->f; a.status = h->dev_small; a.geo = t.es;
         const EsTiles et = es_tile_counts(op.nx, op.ny, op.nz);
         const long tiles = (long)et.kind(0) + et.kind(1);

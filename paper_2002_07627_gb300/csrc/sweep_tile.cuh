@@ -18,6 +18,8 @@ constexpr size_t kSwMaxSmem = 100 * 1024;
 struct SwGeometry {
     int nq = 0, nl = 0, ppw = 0, UP = 0, somax = 0, planes = 0, words = 0;
     size_t smem = 0;
+    // on average per orientation: a thread's shared loads, words a block stages, runs of the cutter along x
+    double cost = 0, stage = 0, runs = 0;
 };
 struct SwOrient {
     int axis;                            // 0: runs along y, planes along z; 1: the other way; -1: no cutter voxels

@@ -97,3 +97,61 @@ def test_tiled_sweep_equals_the_sweep_on_levels(n, r, n_orient, sets):
         imf.close()
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+def _choice(n, tool, nsm=152):
+    """(staged or not, runs of the cutter along x) for one batch of all the tool's orientations on an n = (nx, ny, nz)
+    grid, from the plan that the library makes."""
+    from paper_2002_07627_gb300 import binding, build
+    build.build()
+    imf = binding.Imf(n[::-1], plan_only=True, precision=binding.IMF_FP32_FFT)
+    imf.set_tool(0, tool.holder, tool.cutter, tool.origin, tool.quats)
+    info = imf.tool_info(0)
+    rk = [imf.offsets(0, o, 1) for o in range(info.n_orient)]
+    imf.close()
+    count = np.array([len(v) for v in rk], np.int32)
+    flat = np.ascontiguousarray(np.concatenate(rk), np.int32)
+    K, kmin, runs = np.array(info.kmax, np.int32), flat.min(0).astype(np.int32), ctypes.c_double()
+    L = ctypes.CDLL(build.HOSTLIB)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    got = L.imf_host_sweep_faster(p(flat), p(count), len(count), p(K), p(kmin), *n, nsm, ctypes.byref(runs))
+    want = np.mean([len({(y, z, x) for x, y, z in v.tolist()} - {(y, z, x + 1) for x, y, z in v.tolist()}) for v in rk])
+    assert abs(runs.value - want) <= 1e-9 * want
+    return got
+
+
+@pytest.mark.parametrize("n,r,l,n_orient,want", [
+    ((40, 40, 40), 11, 30, 3, 0), ((40, 40, 40), 11, 30, 32, 0), ((200, 100, 8), 8, 20, 64, 0), ((96, 96, 96), 11, 30, 8, 0),
+    ((128, 128, 128), 11, 30, 32, 0), ((48, 48, 48), 3, 20, 16, 0), ((40, 40, 40), 1, 1, 8, 0), ((128, 128, 128), 3, 20, 64, 1),
+    ((256, 256, 256), 3, 20, 64, 1), ((96, 96, 96), 6, 12, 32, 1), ((400, 60, 32), 11, 3, 64, 1), ((256, 64, 32), 6, 12, 64, 1)])
+def test_the_staged_sweep_is_taken_where_it_measured_faster(n, r, l, n_orient, want):
+    assert _choice(n, synth.cylinder_tool(r, l, r + 3, 8, synth.fibonacci_quats(n_orient))) == want
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,r,l,n_orient", [((97, 70, 67), 4, 9, 48), ((33, 63, 65), 5, 9, 96), ((31, 32, 64), 5, 9, 128),
+                                             ((65, 97, 31), 6, 5, 96), ((20, 40, 160), 6, 5, 64), ((5, 64, 32), 6, 5, 256),
+                                             ((1100, 40, 24), 6, 9, 48)])
+def test_tiled_sweep_equals_the_sweep_on_levels_where_it_runs(n, r, l, n_orient):
+    """As above, on cases that the rule does give to the staged tiles, at word and tile edges."""
+    torch = pytest.importorskip("torch")
+    from paper_2002_07627_gb300 import binding, build
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    tool = synth.cylinder_tool(r, l, r + 2, 5, np.random.default_rng(n_orient).normal(size=(n_orient, 4)))
+    assert _choice(n, tool, torch.cuda.get_device_properties(0).multi_processor_count) == 1
+    rho = torch.from_numpy(synth.beam_density(n, n_beams=6, seed=3)).cuda()
+    got = []
+    for loop in (True, False):
+        imf = binding.Imf(tuple(rho.shape), accessible_by_sweep=True, sweep_loop=loop, orient_batch=n_orient,
+                          precision=binding.IMF_FP32_FFT)
+        imf.set_tools([tool])
+        acc = torch.empty(rho.shape, dtype=torch.uint8, device="cuda")
+        imf.compute(rho, accessible=acc)
+        sets, _, _ = imf.accessible_sets(rho)
+        imf.sync()
+        got.append((acc, sets))
+        imf.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
