@@ -107,8 +107,7 @@ typedef struct {
                                 factor above 16 (same arithmetic, same results): bit 0 = 16
                                 pencils per block or per copy-fed item (128-byte rows) for the z
                                 pass with the spectral product, bit 1 = for the other passes,
-                                else 8 (one-shot or warp-specialised blocks only); -1 = library
-                                default (16 for every pass)                                    */
+                                else 8; -1 = library default (16 for every pass)               */
     int fft_tma;             /* launch form of the two-pass y / z FFT passes (same arithmetic,
                                 same results): bits 0-1 for the z pass with the spectral
                                 product, bits 2-3 for the other passes; 0 = one-shot blocks that

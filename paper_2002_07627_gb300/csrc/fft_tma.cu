@@ -115,7 +115,7 @@ bool launch_axis2_tma(int sign, const AxisArgs &a, int nbatch, int norient, cuda
     const bool ws = a.tma == 2;            // warp-specialised: 8 pencils per item for both shapes
     // big factors: 16 pencils per item (128-byte rows per copy) where the option asks for it
     const bool wide = a.mul ? (a.wide & 1) != 0 : (a.wide & 2) != 0;
-    const int W = ws ? 8 : big ? (wide ? 16 : 8) : 16;
+    const int W = pencils(big, ws, wide);
     const int L = a.A2 * a.B2;
     if (!big && L < kMinLength) return false;
     Params P{};

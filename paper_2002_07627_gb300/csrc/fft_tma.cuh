@@ -48,6 +48,12 @@ bool encode_tiled_u32(CUtensorMap *m, const void *ptr, int rank, const uint64_t 
 // tiny grids, keep the one-shot kernel; fewer instances keep the build short)
 constexpr int kMinLength = 64;
 
+// Pencils per item: 8 for warp-specialised blocks, 16 otherwise, except that passes with a factor above 16 take
+// what the option asks for (16 of them are 128-byte rows a copy, 8 leave room for longer pencils).
+__host__ __device__ constexpr int pencils(bool big, bool ws, bool wide) { return ws || (big && !wide) ? 8 : 16; }
+// which of these fft_tma_inst.cu compiles a launch for
+__host__ __device__ constexpr bool compiled(bool big, bool ws, int W) { return ws ? W == 8 : W == 16 || (big && W == 8); }
+
 struct Params {
     AxisArgs a;
     int axis_is_plane;   // 1: the FFT axis is the plane dimension of the tensor (z pass), 0: rows

@@ -24,8 +24,12 @@ bool IMF_TMA_NAME(const CUtensorMap &in_map, const CUtensorMap &mul_map, Params 
     constexpr int S = IMF_TMA_VARIANT == 0 ? -1 : 1;
     constexpr int MUL = IMF_TMA_VARIANT == 2 ? 1 : 0;
     constexpr bool BIG = IMF_TMA_BIG != 0;
-    if (ws) return W == 8 && launch_ws<S, BIG, MUL, 8>(in_map, mul_map, P, s);
-    return W == 16 && launch_shape<S, BIG, MUL, 16>(in_map, mul_map, P, s);
+    if (!compiled(BIG, ws, W)) return false;
+    if (ws) return launch_ws<S, BIG, MUL, 8>(in_map, mul_map, P, s);
+    if constexpr (compiled(BIG, false, 8)) {
+        if (W == 8) return launch_shape<S, BIG, MUL, 8>(in_map, mul_map, P, s);
+    }
+    return launch_shape<S, BIG, MUL, 16>(in_map, mul_map, P, s);
 }
 
 } // namespace tma_fft

@@ -14,6 +14,7 @@
 #include "erode_plan.h"
 #include "erode_stream.h"
 #include "fft_plan.h"
+#include "fft_tma.cuh"
 #include "grid_barrier.cuh"
 #include "orient_order.h"
 #include "sweep_bits.cuh"
@@ -328,4 +329,11 @@ extern "C" int imf_host_sweep_faster(const int *rk, const int *count, int n_orie
         if (e.axis >= 0) ++kind[e.axis];
     *runs = g.runs;
     return imf::sw_faster(g, nx, ny, nz, kind, n_orient, nsm);
+}
+
+// Pencils per item of the copy-fed y and z passes (fft_tma.cuh), negative where no launch is compiled for them.
+extern "C" int imf_host_tma_pencils(int big, int ws, int wide)
+{
+    const int W = imf::tma_fft::pencils(big != 0, ws != 0, wide != 0);
+    return imf::tma_fft::compiled(big != 0, ws != 0, W) ? W : -W;
 }
