@@ -1206,9 +1206,7 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
                     vbytes((size_t)t.P[2], 8) + vbytes(rto.size(), 4) + vbytes(rts.size(), 4) +
                     vbytes(ivv.size(), sizeof(int4)) + vbytes(ivst.size(), 4) +
                     vbytes(chunks.size(), sizeof(ErodeChunk)) + vbytes(chst.size(), 4) +
-                    vbytes(eruns.size(), sizeof(int2)) + vbytes(t.perm.size(), 4) +
-                    vbytes(es_head.size(), sizeof(EsOrient)) + vbytes(es_words.size(), 4) +
-                    vbytes(sw_head.size(), sizeof(SwOrient)) + vbytes(sw_words.size(), 4);
+                    vbytes(eruns.size(), sizeof(int2)) + vbytes(t.perm.size(), 4);
     if (!plan_only) {
         twiddles(t.M, t.M, t.M, tw);
         if ((st = upload(h, &t.twM, tw))) return bail(st);
@@ -1221,9 +1219,7 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
         if ((st = upload(h, &t.rt_off, rto)) || (st = upload(h, &t.rt_start, rts)) ||
             (st = upload(h, &t.sw_pairs, ivv)) || (st = upload(h, &t.sw_start, ivst)) ||
             (st = upload(h, &t.er_chunks, chunks)) || (st = upload(h, &t.er_chunk_start, chst)) ||
-            (st = upload(h, &t.er_runs, eruns)) || (st = upload(h, &t.perm_dev, t.perm)) ||
-            (st = upload(h, &t.es_head, es_head)) || (st = upload(h, &t.es_words, es_words)) ||
-            (st = upload(h, &t.sw_head, sw_head)) || (st = upload(h, &t.sw_words, sw_words)))
+            (st = upload(h, &t.er_runs, eruns)) || (st = upload(h, &t.perm_dev, t.perm)))
             return bail(st);
     }
     // --- direct tensor-core path: groups, union taps, B matrices
@@ -1239,6 +1235,36 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
     if (prec == IMF_BF16_DIRECT && !t.dir_ok)
         return bail(fail(h, IMF_ERR_INVALID_ARG, "tool too large for the direct tensor-core path"));
     t.path = prec == IMF_BF16_DIRECT ? IMF_BF16_DIRECT : IMF_FP32_FFT;
+    const size_t per = (size_t)t.P[2] * t.P[1] * t.Hs;     // complex values of one tool spectrum
+    // --- tables of the streamed minimum and the staged sweep. Both have other kernels to fall back on, so a budget that
+    // has no room for them beside what the tool cannot do without (its other tables and spectra, the buffers of its
+    // set-up and of a first compute with the fewest slots) leaves them out, as it does where they would take more
+    // than a 64th of what is left over for further tools and slots.
+    const size_t variant_bytes = vbytes(es_head.size(), sizeof(EsOrient)) + vbytes(es_words.size(), 4) +
+                                 vbytes(sw_head.size(), sizeof(SwOrient)) + vbytes(sw_words.size(), 4);
+    if (h->opt.hbm_budget_bytes) {
+        const bool fft = prec != IMF_BF16_DIRECT;
+        const int n_tools = h->n_tools;
+        h->n_tools = std::max(n_tools, tool_id + 1);
+        const WorkSizes ws = work_sizes(h);
+        // ensure_work asks for the slots' shares of the near-threshold list beside its least size
+        const size_t work = h->f ? 0 : work_bytes(h, ws, ws.min_slots) + ws.min_slots * (ws.gn / 32 + 1) * sizeof(int2);
+        h->n_tools = n_tools;
+        // the rest of this tool's tables is on the handle already unless the handle only plans
+        const size_t need = h->owned_bytes + (plan_only ? t.table_bytes : 0) + (fft ? per * n_orient * sizeof(float2) : 0) +
+                            std::max(work, fft ? (size_t)t.P[0] * t.P[1] * t.P[2] * 4 + 2 * per * sizeof(float2) : 0);
+        const size_t room = h->opt.hbm_budget_bytes > need ? h->opt.hbm_budget_bytes - need : 0;
+        if (variant_bytes > room / 64) {
+            t.es_ok = t.sw_ok = false;
+            es_head.clear(); es_words.clear(); sw_head.clear(); sw_words.clear();
+        }
+    }
+    if (t.es_ok || t.sw_ok) {
+        t.table_bytes += variant_bytes;
+        if (!plan_only && ((st = upload(h, &t.es_head, es_head)) || (st = upload(h, &t.es_words, es_words)) ||
+                           (st = upload(h, &t.sw_head, sw_head)) || (st = upload(h, &t.sw_words, sw_words))))
+            return bail(st);
+    }
     if (prec == IMF_BF16_DIRECT) {
         t.setup_bytes = std::max(rot_bytes, t.table_bytes);
         t.planned_only = plan_only;
@@ -1248,7 +1274,6 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
     }
 
     // --- tool spectra: conj(FFT(1_RT)) / Ptot (reflection as conjugation, Alg. 1 footnote)
-    const size_t per = (size_t)t.P[2] * t.P[1] * t.Hs;
     t.spec_bytes = per * n_orient * sizeof(float2);
     // transient buffers of the spectrum build: the dense padded tool and two intermediates
     t.setup_bytes = std::max(rot_bytes, t.table_bytes + t.spec_bytes + (size_t)t.P[0] * t.P[1] * t.P[2] * 4 +

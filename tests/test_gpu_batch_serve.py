@@ -212,3 +212,38 @@ def test_clone_shares_tools_and_outlives_its_parent():
     c.sync()
     assert np.array_equal(x.cpu().numpy(), ref[0]) and np.array_equal(y.cpu().numpy(), ref[1])
     c.close()
+
+
+@pytest.mark.parametrize("n_orient", [1, 24])
+def test_a_budget_without_room_for_the_optional_tables_is_enough(n_orient):
+    """One byte less than a tool takes with one slot and the tables of the streamed minimum and the staged sweep (the
+    planned figure and the slot's share of the near-threshold list): those are left out, and results do not depend
+    on them."""
+    _need_gpu()
+    from paper_2002_07627_gb300 import binding, synth
+    shape = (70, 45, 64)
+    rho = torch.from_numpy(synth.beam_density(shape[::-1], n_beams=6, seed=1)).cuda()
+    tool = synth.cylinder_tool(3, 12, 6, 8, synth.fibonacci_quats(n_orient))
+
+    def run(budget):
+        imf = binding.Imf(shape, hbm_budget_bytes=budget, precision=binding.IMF_FP32_FFT, accessible_by_sweep=True)
+        imf.set_tools([tool])
+        acc = torch.empty(shape, dtype=torch.uint8, device="cuda")
+        raw = torch.empty_like(rho)
+        fb, sec = imf.compute(rho, raw=raw, accessible=acc)
+        imf.sync()
+        owned = imf.stats().owned_bytes
+        imf.close()
+        return (fb, sec, raw, acc), owned
+
+    plan = binding.Imf(shape, plan_only=True, precision=binding.IMF_FP32_FFT, accessible_by_sweep=True)
+    plan.set_tools([tool])
+    fp, win = plan.footprint(1), plan.tool_info(0).win
+    plan.close()
+    full, _ = run(0)
+    share = ((win[0] + 3) // 4 * 4 * win[1] * win[2] // 32 + 1) * 8
+    tight = max(int(fp.resident + fp.work) + share, int(fp.setup_peak)) - 1
+    got, owned = run(tight)
+    assert owned <= tight
+    for a, b in zip(full, got):
+        assert torch.equal(a, b)
