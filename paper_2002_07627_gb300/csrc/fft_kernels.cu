@@ -9,6 +9,8 @@
 // it loads (the pointwise product of App. B), and the inverse x pass writes the collision
 // measure g together with the bit mask of collision-free translations (threshold of
 // Eq. eq_conv_D) and the list of translations whose g lies within the re-check band.
+#include <type_traits>
+
 #include "imf_internal.cuh"
 #include "threshold_row.cuh"
 
@@ -57,11 +59,11 @@ __device__ void run_stages(const FftPlan &plan, float2 *&src, float2 *&dst, int 
     }
 }
 
-constexpr int kAxisW = 16;
-
-template <int S>
+// A block holds W = 2^LOGW pencils: 16 (128-byte segments), or as many of them as fit shared memory (launch_axis_fft)
+template <int S, int LOGW>
 __global__ void __launch_bounds__(kThreads) axis_fft_kernel(AxisArgs a)
 {
+    constexpr int kAxisW = 1 << LOGW;
     extern __shared__ float2 sm[];
     const int L = a.plan.L;
     float2 *buf0 = sm, *buf1 = sm + kAxisW * L, *tw = sm + 2 * kAxisW * L;
@@ -94,7 +96,7 @@ __global__ void __launch_bounds__(kThreads) axis_fft_kernel(AxisArgs a)
     }
     __syncthreads();
     float2 *src = buf0, *dst = buf1;
-    run_stages<S, 4>(a.plan, src, dst, kAxisW, tw);
+    run_stages<S, LOGW>(a.plan, src, dst, kAxisW, tw);
     float2 *out = a.out + o * a.out_so + b * a.out_sb + kx0;
     for (int idx = threadIdx.x; idx < kAxisW * a.lout; idx += blockDim.x) {
         const int w = idx % kAxisW, jj = idx / kAxisW;
@@ -219,15 +221,36 @@ template <typename K> void set_smem(K kernel, size_t bytes)
     if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-// rows per x-pass block: 32 while the two staging buffers stay near 100 KB, else 16 or 8
+constexpr size_t kMaxSmem = 227 * 1024;
+
+size_t axis_smem(int L, int W) { return (size_t)(2 * W + 1) * L * sizeof(float2); }
+size_t x_smem(int M, int W) { return (size_t)(2 * (M + 1) * (W + 1) + 2 * M + 1) * sizeof(float2); }
+
+// pencils per axis-pass block (log2): 16, fewer above length 880 (two at make_plan's limit of 4096)
+int axis_log_pencils(int L)
+{
+    int lw = 4;
+    while (lw > 0 && axis_smem(L, 1 << lw) > kMaxSmem) --lw;
+    return lw;
+}
+
+// rows per x-pass block (log2): 32 while the two staging buffers stay near 100 KB, else 16, 8, or as many as fit
+// (fewer than 8 above M = 1452, one at make_plan's limit of 4096)
 int x_log_rows(int M)
 {
     if ((size_t)(M + 1) * 33 * 16 <= 100 * 1024) return 5;
     if ((size_t)(M + 1) * 17 * 16 <= 100 * 1024) return 4;
-    return 3;
+    int lw = 3;
+    while (lw > 0 && x_smem(M, 1 << lw) > kMaxSmem) --lw;
+    return lw;
 }
 
-size_t x_smem(int M, int W) { return (size_t)(2 * (M + 1) * (W + 1) + 2 * M + 1) * sizeof(float2); }
+// f(LOGW as a constant) for lw in [0, N]
+template <int N, typename F> void with_log(int lw, F &&f)
+{
+    if (lw == N) f(std::integral_constant<int, N>{});
+    else if constexpr (N > 0) with_log<N - 1>(lw, f);
+}
 
 } // namespace
 
@@ -237,15 +260,17 @@ void launch_axis_fft(int sign, const AxisArgs &a, int nbatch, int norient, cudaS
         launch_axis2(sign, a, nbatch, norient, s);
         return;
     }
-    const size_t smem = (size_t)(2 * kAxisW * a.plan.L + a.plan.L) * sizeof(float2);
-    dim3 grid((a.nx + kAxisW - 1) / kAxisW, nbatch, norient);
-    if (sign < 0) {
-        set_smem(axis_fft_kernel<-1>, smem);
-        axis_fft_kernel<-1><<<grid, kThreads, smem, s>>>(a);
-    } else {
-        set_smem(axis_fft_kernel<1>, smem);
-        axis_fft_kernel<1><<<grid, kThreads, smem, s>>>(a);
-    }
+    with_log<4>(axis_log_pencils(a.plan.L), [&](auto LW) {
+        constexpr int W = 1 << decltype(LW)::value;
+        const size_t smem = axis_smem(a.plan.L, W);
+        const dim3 grid((a.nx + W - 1) / W, nbatch, norient);
+        auto go = [&](auto kernel) {
+            set_smem(kernel, smem);
+            kernel<<<grid, kThreads, smem, s>>>(a);
+        };
+        if (sign < 0) go(axis_fft_kernel<-1, decltype(LW)::value>);
+        else go(axis_fft_kernel<1, decltype(LW)::value>);
+    });
 }
 
 void launch_rfft_fwd(const RfftArgs &a, cudaStream_t s)
@@ -253,12 +278,12 @@ void launch_rfft_fwd(const RfftArgs &a, cudaStream_t s)
     // fewer rows a block where 32 of them would leave SMs without one (same arithmetic per row)
     int lw = x_log_rows(a.M);
     while (lw > 3 && (a.rows >> lw) < 2 * 152) --lw;
-    const int W = 1 << lw;
-    const size_t smem = x_smem(a.M, W);
-    dim3 grid((a.rows + W - 1) / W);
-    if (lw == 5) { set_smem(rfft_fwd_kernel<5>, smem); rfft_fwd_kernel<5><<<grid, kThreads, smem, s>>>(a); }
-    else if (lw == 4) { set_smem(rfft_fwd_kernel<4>, smem); rfft_fwd_kernel<4><<<grid, kThreads, smem, s>>>(a); }
-    else { set_smem(rfft_fwd_kernel<3>, smem); rfft_fwd_kernel<3><<<grid, kThreads, smem, s>>>(a); }
+    with_log<5>(lw, [&](auto LW) {
+        constexpr int W = 1 << decltype(LW)::value;
+        const size_t smem = x_smem(a.M, W);
+        set_smem(rfft_fwd_kernel<decltype(LW)::value>, smem);
+        rfft_fwd_kernel<decltype(LW)::value><<<dim3((a.rows + W - 1) / W), kThreads, smem, s>>>(a);
+    });
 }
 
 void launch_irfft_threshold(const IrfftArgs &a, int norient, cudaStream_t s)
@@ -267,12 +292,12 @@ void launch_irfft_threshold(const IrfftArgs &a, int norient, cudaStream_t s)
         launch_irfft2_threshold(a, norient, s);
         return;
     }
-    const int lw = x_log_rows(a.M), W = 1 << lw;
-    const size_t smem = x_smem(a.M, W);
-    dim3 grid((a.rows + W - 1) / W, 1, norient);
-    if (lw == 5) { set_smem(irfft_threshold_kernel<5>, smem); irfft_threshold_kernel<5><<<grid, kThreads, smem, s>>>(a); }
-    else if (lw == 4) { set_smem(irfft_threshold_kernel<4>, smem); irfft_threshold_kernel<4><<<grid, kThreads, smem, s>>>(a); }
-    else { set_smem(irfft_threshold_kernel<3>, smem); irfft_threshold_kernel<3><<<grid, kThreads, smem, s>>>(a); }
+    with_log<5>(x_log_rows(a.M), [&](auto LW) {
+        constexpr int W = 1 << decltype(LW)::value;
+        const size_t smem = x_smem(a.M, W);
+        set_smem(irfft_threshold_kernel<decltype(LW)::value>, smem);
+        irfft_threshold_kernel<decltype(LW)::value><<<dim3((a.rows + W - 1) / W, 1, norient), kThreads, smem, s>>>(a);
+    });
 }
 
 } // namespace imf
