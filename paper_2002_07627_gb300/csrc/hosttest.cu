@@ -16,6 +16,7 @@
 #include "fft_plan.h"
 #include "fft_tma.cuh"
 #include "grid_barrier.cuh"
+#include "launch_errors.h"
 #include "orient_order.h"
 #include "sweep_bits.cuh"
 #include "sweep_plan.h"
@@ -336,4 +337,15 @@ extern "C" int imf_host_tma_pencils(int big, int ws, int wide)
 {
     const int W = imf::tma_fft::pencils(big != 0, ws != 0, wide != 0);
     return imf::tma_fft::compiled(big != 0, ws != 0, W) ? W : -W;
+}
+
+// Feeds n launch results to a call's record; returns what the call reports with `last` as the runtime's final word, and
+// in next what a following call without errors reports.
+extern "C" int imf_host_launch_errors(const int *results, int n, int last, int *next)
+{
+    imf::LaunchErrors e;
+    for (int i = 0; i < n; ++i) e.note((cudaError_t)results[i]);
+    const int got = (int)e.take((cudaError_t)last);
+    *next = (int)e.take(cudaSuccess);
+    return got;
 }

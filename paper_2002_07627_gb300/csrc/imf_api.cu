@@ -29,6 +29,7 @@
 #include "erode_plan.h"
 #include "erode_stream.h"
 #include "fft_plan.h"
+#include "launch_errors.h"
 #include "orient_order.h"
 #include "sweep_plan.h"
 
@@ -161,6 +162,7 @@ struct imf_handle_s {
     bool used_stream = false;
     size_t owned_bytes = 0;
     std::unordered_map<void *, size_t> sizes;
+    LaunchErrors launch_errors;
     // stats
     long launches = 0, computes = 0, flagged_last = 0, flagged_total = 0;
     // profiling
@@ -269,6 +271,7 @@ struct Launch {
     cudaEvent_t a = nullptr;
     Launch(imf_handle h_, int kid_, cudaStream_t s_) : h(h_), kid(kid_), s(s_)
     {
+        cudaGetLastError();              // what an earlier call left, and reported
         if (h->prof) {
             a = get_event(h);
             cudaEventRecord(a, s);
@@ -276,6 +279,7 @@ struct Launch {
     }
     ~Launch()
     {
+        h->launch_errors.note(cudaGetLastError());
         h->launches++;
         if (h->prof) {
             cudaEvent_t b = get_event(h);
@@ -958,6 +962,7 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
     if (h->tool_refs && h->tool_refs.use_count() > 1)
         return fail(h, IMF_ERR_INVALID_ARG, "the tools of this handle are shared with a clone (imf_clone)");
     if (h->used_stream) CU(cudaStreamSynchronize(h->last_stream));
+    h->launch_errors = LaunchErrors{};
     Tool &t = h->tools[tool_id];
     if (t.set) free_tool(h, t);
     t.tx = tx; t.ty = ty; t.tz = tz;
@@ -1033,6 +1038,7 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
         }
         hout.resize((size_t)tot * 3);
         cudaError_t e = cudaMemcpy(hout.data(), dout, (size_t)tot * 3, cudaMemcpyDeviceToHost);
+        e = h->launch_errors.take(e);
         cleanup();
         if (e != cudaSuccess) return fail(h, IMF_ERR_CUDA, "rotate: %s", cudaGetErrorString(e));
     }
@@ -1303,6 +1309,7 @@ imf_status imf_set_tool(imf_handle h, int tool_id, const uint8_t *holder, const 
         st = forward_real_3d(h, t, dense, nullptr, t.P[0], t.P[1], t.P[2], s1, s2, t.spec + per * i, (float)(1.0 / ptot), 1, 0);
     }
     cudaError_t e = cudaDeviceSynchronize();
+    e = h->launch_errors.take(e);
     dfree(h, dense, dn); dfree(h, s1, per); dfree(h, s2, per);
     if (st != IMF_OK) return bail(st);
     if (e != cudaSuccess) return bail(fail(h, IMF_ERR_CUDA, "tool spectrum: %s", cudaGetErrorString(e)));
@@ -1427,6 +1434,7 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
 {
     const imf_options &op = h->opt;
     const long N = (long)op.nx * op.ny * op.nz;
+    h->launch_errors = LaunchErrors{};
     TRY(ensure_work(h));
     if (!h->f || !h->A || !h->dev_small || !h->flags || !h->Y1 || !h->Y2 || !h->g || !h->bits || !h->rho_spec ||
         !h->X1 || !h->X2 || h->slots < 1)
@@ -1575,7 +1583,7 @@ static imf_status compute_impl(imf_handle h, const float *rho, const uint8_t *fi
         if (small_grid(N)) launch_finalize_small(a, s);
         else launch_finalize(a, s);
     }
-    CU(cudaGetLastError());
+    CU(h->launch_errors.take(cudaGetLastError()));
     h->computes++;
     return IMF_OK;
 }
@@ -1625,6 +1633,7 @@ imf_status imf_penalize_sensitivity(imf_handle h, float *sens, const float *rho_
     if (!(w_acc >= 0.0 && w_acc < 1.0)) return fail(h, IMF_ERR_INVALID_ARG, "w_acc %g outside [0, 1)", w_acc);
     const long N = (long)h->opt.nx * h->opt.ny * h->opt.nz;
     cudaStream_t s = (cudaStream_t)cuda_stream;
+    h->launch_errors = LaunchErrors{};
     TRY(ensure_small(h));
     unsigned *mb = (unsigned *)(h->dev_small + 3);
     h->last_stream = s;
@@ -1642,7 +1651,7 @@ imf_status imf_penalize_sensitivity(imf_handle h, float *sens, const float *rho_
         Launch L(h, KID_PENALIZE, s);
         launch_penalize(sens, rho_omega, imf_bar, secluded, N, mb, (unsigned *)(h->dev_small + 5), w_acc, h->opt.tau, s);
     }
-    CU(cudaGetLastError());
+    CU(h->launch_errors.take(cudaGetLastError()));
     return IMF_OK;
 }
 
@@ -1678,6 +1687,7 @@ imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, cons
     const long awords = (op.nx + 31) / 32;
     const long words = (long)op.nz * op.ny * awords;
     cudaStream_t s = (cudaStream_t)cuda_stream;
+    h->launch_errors = LaunchErrors{};
     if (2 * (size_t)words > h->plan_rem_n) {
         dfree(h, h->plan_rem);
         h->plan_rem_n = 0;
@@ -1714,6 +1724,7 @@ imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, cons
     std::vector<long long> out(need - nc);
     CU(cudaMemcpyAsync(out.data(), h->plan_cnt + nc, out.size() * sizeof(long long), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
+    CU(h->launch_errors.take(cudaGetLastError()));
     unsigned bar[2];
     std::memcpy(bar, out.data(), sizeof bar);
     if (bar[1]) return fail(h, IMF_ERR_TIMEOUT, "process plan: a grid barrier timed out");
