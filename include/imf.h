@@ -125,14 +125,15 @@ typedef struct {
                                 (planes too large for the fused y + x pass): 1 = persistent
                                 blocks fed by tensor copies of whole rows, 0 = one-shot blocks;
                                 same results; -1 = library default (1)                        */
-    int sweep_loop;          /* the sweep of Eq. eq_conv_A: 0 (default) = one thread per output
-                                word and orientation of the batch; 1 = each thread walks the
-                                batch's orientations for its word and stops once the word is
+    int sweep_loop;          /* the sweep of Eq. eq_conv_A: 0 (default) = staged tiles where they
+                                are estimated to be faster, else one thread per output word and
+                                orientation of the batch on dilation levels; 1 = each thread walks
+                                the batch's orientations for its word and stops once the word is
                                 fully accessible (same results; slower where measured)         */
     int erode_xt;            /* minimum over sharp points: 8 or 16 = the tiled kernel with that many
                                 consecutive x outputs per thread (1024 or 512 threads per block);
-                                same results; 0 = library default: the streamed kernel for 3D
-                                grids with work enough for it, else the tiled one with 8      */
+                                same results; 0 = library default: the streamed kernel in 3D
+                                where it is estimated to be faster, else the tiled one with 8 */
 } imf_options;
 
 /* Fill *opt with the defaults above (grid 0x0x0, which imf_create rejects). */
@@ -241,7 +242,8 @@ imf_status imf_compute_accessible_sets(imf_handle h, const float *rho_omega, con
  *   n_steps    : HOST out, steps taken; negative / left (or NULL): HOST out, |N| and the
  *                voxels no set can reach (inaccessible negative space).
  * Synchronous (one launch). Uses handle-owned scratch (grown on demand).
- * Errors: IMF_ERR_INVALID_ARG (NULL, n_sets < 1, max_steps < 0), IMF_ERR_OOM, IMF_ERR_CUDA. */
+ * Errors: IMF_ERR_INVALID_ARG (NULL, n_sets < 1, max_steps < 0), IMF_ERR_OOM, IMF_ERR_BUDGET, IMF_ERR_CUDA,
+ * IMF_ERR_TIMEOUT (the launch's blocks waited for each other for more than five seconds). */
 imf_status imf_process_plan(imf_handle h, const uint32_t *sets, int n_sets, const float *rho_omega,
                             const uint8_t *fixture, int max_steps, int *order, long long *removed, int *n_steps,
                             long long *negative, long long *left, void *cuda_stream);

@@ -6,7 +6,9 @@
  *
  *   Heaviside projection (Eq. eq_Heaviside): rho = 1 - exp(-beta xi) + xi exp(-beta);
  *   FEA: bilinear four-node plane-stress elements, SIMP modulus E(rho) = Emin + rho^p (E0 - Emin),
- *        K(rho) u = f solved by a matrix-free Jacobi-preconditioned conjugate gradient in FP64;
+ *        K(rho) u = f solved by a conjugate gradient in FP64 on the assembled node stencil, with a
+ *        multigrid V-cycle in FP32 as its preconditioner (or, where that stalls, matrix-free with the
+ *        diagonal as preconditioner);
  *   compliance c = f^T u and its sensitivity to xi (self-adjoint, Sec. 2.2), smoothed by a
  *        mesh-independence filter (hat weights max(0, rmin - distance));
  *   optimality-criteria update of xi with a move limit and the volume constraint on the
@@ -47,7 +49,8 @@ typedef struct {
  * cg_max_iter = 20000 (grid 0 x 0, which imf_to2d_create rejects). */
 void imf_to2d_default_options(imf_to2d_options *opt);
 
-/* Allocates the solver vectors. Errors: IMF_ERR_INVALID_ARG, IMF_ERR_OOM. */
+/* Allocates the solver vectors, about 112 bytes a node, and the multigrid hierarchy, about 530 more, where that is
+ * at most 256 MB or a sixteenth of the free memory. Errors: IMF_ERR_INVALID_ARG, IMF_ERR_OOM. */
 imf_status imf_to2d_create(const imf_to2d_options *opt, imf_to2d *out);
 void imf_to2d_destroy(imf_to2d h);
 const char *imf_to2d_last_error(imf_to2d h);
@@ -74,12 +77,13 @@ imf_status imf_to2d_analyze(imf_to2d h, const float *rho, const double *force, c
 imf_status imf_to2d_sensitivity(imf_to2d h, const float *xi, const float *rho, float *sens, void *cuda_stream);
 
 /* Optimality-criteria update xi_new = clamp(xi (S / lam)^eta) within [xi - move, xi + move] and
- * [0, 1], lam by bisection so that the mean projected density of the non-passive elements is
- * volfrac; passive elements (DEVICE uint8, or NULL) keep xi = 1. S: DEVICE float, >= 0.
+ * [0, 1], lam by bracketed Newton steps so that the mean projected density of the non-passive elements
+ * is volfrac; passive elements (DEVICE uint8, or NULL) keep xi = 1. S: DEVICE float, >= 0.
  * change_out (HOST, or NULL) receives the mean |xi_new - xi| over the non-passive elements
  * (Alg. 2's volume difference), vol_out (HOST, or NULL) the mean projected density reached.
  * Synchronous (one launch; eta above 4 takes a bisection on the host, one volume reduction per step).
- * Errors: IMF_ERR_INVALID_ARG (NULL, volfrac outside (0, 1), move <= 0), IMF_ERR_CUDA. */
+ * Errors: IMF_ERR_INVALID_ARG (NULL, volfrac outside (0, 1), move <= 0), IMF_ERR_CUDA, IMF_ERR_TIMEOUT (the
+ * launch's blocks waited for each other for more than five seconds). */
 imf_status imf_to2d_update(imf_to2d h, const float *xi, const float *S, const uint8_t *passive, double volfrac,
                            double move, double eta, float *xi_new, double *change_out, double *vol_out,
                            void *cuda_stream);

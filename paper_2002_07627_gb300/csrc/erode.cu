@@ -17,8 +17,8 @@
 // an integer atomic minimum, which orders non-negative floats (every g >= 0; -0 is mapped to +0
 // first) exactly as the float minimum does, so the result does not depend on the split.
 //
-// Large 3D grids take erode_stream.cu instead (imf_api.cu holds the rule); this kernel serves planar grids,
-// grids of few tiles, where it is as fast or faster, and the forms that the options choose.
+// 3D batches whose estimate is lower there take erode_stream.cu instead (es_faster in erode_stream.h); this kernel
+// serves planar grids, few tiles or cheap cutters, and the forms that the options choose.
 #include <cfloat>
 
 #include "erode.cuh"

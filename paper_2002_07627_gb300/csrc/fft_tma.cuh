@@ -12,13 +12,15 @@
 // Two stages alternate: the copy of the block's next item is in flight while this one is transformed. What
 // bounds a pass is how many items an SM has in hand (barriers and waits of one block leave the SM to the others)
 // and how many bytes it has in flight. Each split (A, B) is its own kernel with 16 A threads, so that its registers
-// are its own (one kernel with every split inside took the largest one's, 112 to 124). For lengths up to 256 the
-// tile between the two DFT passes lies in the item's own stage, which pass 1 has read into registers by then: two
-// to four blocks an SM, where a tile buffer left room for one with the factor. Above 256 one block with a tile of its
-// own stays: two with the tile in the stage took 11.2 ms for the 256^3 y pass against 6.0 (a single stage a
+// are its own (one kernel with every split inside took the largest one's, 112 to 124). Where both factors are at most
+// 16 (lengths up to 256, but not 147, 162, 189, 200, 216 or 252, which split into larger ones) the tile between the two
+// DFT passes lies in the item's own stage, which pass 1 has read into registers by then: two to four blocks an SM,
+// where a tile buffer left room for one with the factor. With a larger factor one block with a tile of its own stays: two with the tile in the stage took 11.2 ms for the 256^3 y pass against 6.0 (a single stage a
 // block likewise, 11.5 and 10.8 for the z pass against 7.2). Measured, ms a step, against one kernel per shape:
 // z pass with the factor 128^3 x 64 0.787 -> 0.694, 144^3 x 96 1.70 -> 1.52, 75 x 61 x 50 x 24 0.090 -> 0.063, 48^3 x 24 0.068 ->
-// 0.047; 256^3 x 128 z 7.40 -> 7.25, y 6.18 -> 5.98.
+// 0.047; 256^3 x 128 z 7.40 -> 7.25, y 6.18 -> 5.98. The inverse passes without the factor are held to 80 registers
+// and some spill there (16 x 15: 80 bytes); over lengths 64 to 420 none is slower for it than one kernel per shape was
+// (8 orientations, us: 240 35.0 -> 29.6, 224 33.2 -> 28.7, 210 33.5 -> 27.8).
 //
 // Every wait on a copy is bounded (%globaltimer); on a timeout the block records
 // IMF_ERR_TIMEOUT in the status word, waits (bounded again) for the copies it still has in
@@ -70,7 +72,8 @@ __host__ __device__ constexpr int min_blocks(int W, int A, int B, bool mul)
 {
     if (A > fft2::kMaxFactor) return 1;
     const int smem = kStages * A * B * W * 8 * (mul ? 2 : 1) + A * B * 8 + 512, by_smem = 220 * 1024 / smem;
-    // the warps of n blocks spread over four partitions of 512 registers a lane each, 80 a thread
+    // the warps of n blocks spread over four partitions of 512 registers a lane each, 80 a thread (the compiler
+    // keeps to that; see above for what it costs)
     int n = by_smem < 6 ? by_smem : 6;
     while (n > 1 && (n * threads(W, A) / 32 + 3) / 4 * 80 > 512) --n;
     return n < 1 ? 1 : n;
@@ -105,7 +108,7 @@ __device__ __forceinline__ void issue_item(const Params &P, const void *in_map, 
     }
 }
 
-// where the tile between the passes lies: in the item's own stage (lengths up to 256), or in a buffer of its own
+// where the tile between the passes lies: in the item's own stage (factors up to 16), or in a buffer of its own
 __host__ __device__ constexpr bool tile_in_stage(int A) { return A <= fft2::kMaxFactor; }
 
 // One split L = NA NB: the persistent loop over this block's items.

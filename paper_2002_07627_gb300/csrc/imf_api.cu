@@ -1413,7 +1413,10 @@ imf_status tail_batch(imf_handle h, const Tool &t, const float *rho, const uint8
         a.planar = t.erode_planar;
         // (tile, orientation group) units: at least about twelve waves of resident blocks and
         // at most 16 orientations per block (measured optimum: 8 groups of 8 orientations at
-        // 128^3 x 64, 4 groups of 16 at 256^3 with 64 orientations per launch)
+        // 128^3 x 64, 4 groups of 16 at 256^3 with 64 orientations per launch). Planar blocks are counted as if they were
+        // the 3D ones, half as high and one an SM: counted as they are (64 x 32, four an SM) the rule asks for four
+        // times the groups, which is slower on large grids (us, so and with that many groups: 2048^2 x 16 268 and 313,
+        // 1024^2 x 8 56.8 and 89.8) and changes nothing on small ones, which have a group for every orientation
         const long tiles = (long)((op.nx + kErTX - 1) / kErTX) * ((op.ny + kErTY - 1) / kErTY) *
                            ((op.nz + kErTZ - 1) / kErTZ);
         const long slots = (long)t.erode_bps * h->nsm;

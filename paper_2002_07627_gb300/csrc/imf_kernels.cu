@@ -87,8 +87,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 // sliding OR of length L = b - a + 1 of one source row. With the dilation levels
 // D_j(i) = OR_{t < 2^j} free(i + t) (D_0 = free), the sliding OR of length L at i is
 // D_j(i) | D_j(i + L - 2^j) for 2^j <= L <= 2^(j+1), so every run costs two 32-bit windows.
-// Tools whose cutter fits the plan of staged tiles run sweep_tile.cu instead; this is the route of the others
-// and of the sweep_loop option.
+// Batches whose estimate is lower on staged tiles run sweep_tile.cu instead (sw_faster in sweep_plan.h); this is the
+// route of the others and of the sweep_loop option.
 // ---------------------------------------------------------------------------------------
 
 // Levels 1..4 of the free bits of slots [0, nb): word i of level j at bits + j * lstride + i.

@@ -1,13 +1,12 @@
 // The SIMP steps of the topology-optimisation loop around the IMF (Alg. 2; include/imf_to.h):
-// Heaviside projection, matrix-free FEA with a Jacobi-preconditioned conjugate gradient (FP64),
-// compliance sensitivity with its filter, and the optimality-criteria update.
+// Heaviside projection, FEA, compliance sensitivity with its filter, and the optimality-criteria update.
 //
 // The FEA and the update run as cooperative kernels (topopt2d_mg.cu). What stands here beside the entry
-// points takes over where those do not apply: the Jacobi-preconditioned iteration for designs on which the
-// multigrid-preconditioned one does not converge (or whose hierarchy does not fit), and the host's bisection
-// for exponents whose powers would leave the FP64 range.
+// points takes over where those do not apply: a matrix-free, Jacobi-preconditioned conjugate gradient (FP64) for
+// designs on which the multigrid-preconditioned one stalls (or whose hierarchy does not fit), and the host's
+// bisection for exponents whose powers would leave the FP64 range.
 //
-// The stiffness operator is applied node by node: a node gathers the contributions of its (up
+// That iteration applies the stiffness operator node by node: a node gathers the contributions of its (up
 // to four) elements, E_e times the rows of the element matrix k0 that belong to its corner, so
 // no atomics are needed. The conjugate gradient keeps its scalars on the device (rotating slots,
 // so that a kernel never reads a slot another block of the same launch is resetting); the host

@@ -1,14 +1,14 @@
 // Conjugate gradient with a multigrid preconditioner (geometric V-cycle, Galerkin coarse operators; as
 // Amir, Aage and Lazarov, "On multigrid-CG for efficient topology optimization", 2014, use it) for the FEA
-// of Alg. 2, and the bisection of the optimality-criteria update, each as one cooperative kernel.
+// of Alg. 2, and the optimality-criteria update with its multiplier, each as one cooperative kernel.
 //
 // What bound the plain Jacobi-preconditioned iteration (kept in topopt2d.cu for what this one does not
 // solve): thousands of iterations, each three launches and a few microseconds of FP64 (this part runs
 // two FP64 multiply-adds per SM and clock), with a host round trip every sixteen. On the 256 x 128 cantilever
-// midway in its loop that was 5500 iterations of 24.8 us, 136.8 ms; here 92 of about 50 us, 5.3 ms with the
+// midway in its loop that was 5500 iterations of 24.8 us, 136.8 ms; here 92 of about 55 us, 5.3 ms with the
 // set-up, bound by the grid barriers (eight an iteration) and the latency of the short phases between them.
-// The update's bisection took 36 host round trips, 1.0 ms; in one launch 0.17 ms, and with Newton steps about
-// 0.03 ms, bound by the FP64 exponentials of the projected density and the grid barriers.
+// The update's bisection took 36 host round trips, 1.0 ms; in one launch 0.17 ms, and with Newton steps instead
+// 0.10 ms with the copies, bound by the FP64 exponentials of the projected density and the grid barriers.
 //
 // The iteration itself (operator, vectors, scalar products, stopping rule) is FP64 as before; only the
 // preconditioner, which steers the search directions and not what they converge to, works in FP32: at

@@ -1,5 +1,5 @@
 // Cooperative kernels of the 2D optimisation loop (topopt2d.cu): the multigrid-preconditioned
-// conjugate gradient and the bisection of the optimality-criteria update, each one launch.
+// conjugate gradient and the optimality-criteria update, each one launch.
 #pragma once
 #include <cstddef>
 #include <cstdint>
