@@ -205,20 +205,23 @@ template <int P> struct EsProducer {
     uint64_t *full, *empty;
     int *s_stop;
     uint32_t ring0, stage_bytes;
-    int axis, X0, U0, W0;
-    // the orientation it is at
-    EsOrient h;
-    int ob, cols, rows, gu0;
+    int X0, U0, W0, nu, nw;                // tile origin, window extents along the run and the plane axis
+    long su, sw;                           // strides of g along these
+    // the orientation it is at: columns, rows and first place of what it copies, its first plane, its descriptors
+    int cols, rows, gw0, words, word0;
     const float *src0;
 
     __device__ __forceinline__ int steps(int k)
     {
-        ob = s_ob[k];
-        h = a.head[a.orient_base + ob];
-        gu0 = U0 + h.ou;
+        const int ob = s_ob[k];
+        const EsOrient h = a.head[a.orient_base + ob];
+        const int gu0 = U0 + h.ou, row0 = (threadIdx.x & 31) >> 4;
         cols = min(h.quads, (a.gpx - (X0 + h.ox)) >> 2);       // columns the window's rows have from here
-        rows = min(h.rows, (axis ? a.wz : a.wy) - gu0);
-        src0 = a.g + ob * a.g_so + X0 + h.ox;
+        rows = min(h.rows, nu - gu0);
+        gw0 = W0 + h.ow;
+        words = h.words;
+        word0 = h.word0;
+        src0 = a.g + ob * a.g_so + X0 + h.ox + (gu0 + row0) * su;
         return kEsNW + h.lists;
     }
     __device__ __forceinline__ bool wait(int st, uint32_t phase)
@@ -233,8 +236,8 @@ template <int P> struct EsProducer {
         // the orientation's descriptors; the slot's last readers, four orientations back, gave
         // back their stages at least ten stages ago (an orientation has three or more)
         if (!late)
-            for (int i = tid; i < h.words / 4; i += kEsProducers)
-                reinterpret_cast<int4 *>(s_words + slot * a.geo.words)[i] = __ldg(reinterpret_cast<const int4 *>(a.words + h.word0) + i);
+            for (int i = tid; i < words / 4; i += kEsProducers)
+                reinterpret_cast<int4 *>(s_words + slot * a.geo.words)[i] = __ldg(reinterpret_cast<const int4 *>(a.words + word0) + i);
         // the units that still have work, as one warp sees them; none: the block is done
         if (tid < 32) {
             const uint32_t mask = __ballot_sync(0xffffffffu, ((volatile unsigned char *)s_live)[lane] != 0);
@@ -256,12 +259,10 @@ template <int P> struct EsProducer {
     {
         // a producer warp copies whole planes: 16 lanes a row, two rows a step
         const int tid = threadIdx.x - 32 * kEsWarps, lane = tid & 31, ch = lane & 15, row0 = lane >> 4;
-        const long su = axis ? (long)a.gpx * a.wy : a.gpx, sw = axis ? a.gpx : (long)a.gpx * a.wy;
-        const int nw = axis ? a.wy : a.wz, Q = a.geo.Q, gw0 = W0 + h.ow + 4 * s;
-        for (int pl = tid >> 5; pl < 4 && gw0 + pl < nw; pl += kEsProducers / 32)
+        for (int pl = tid >> 5; pl < 4 && gw0 + 4 * s + pl < nw; pl += kEsProducers / 32)
             for (int c = ch; c < cols; c += 16) {
-                const float *src = src0 + (gw0 + pl) * sw + (gu0 + row0) * su + 4 * c;
-                uint32_t dst = ring0 + st * stage_bytes + 4u * (uint32_t)(pl * Q + row0 * P + 4 * c);
+                const float *src = src0 + (gw0 + 4 * s + pl) * sw + 4 * c;
+                uint32_t dst = ring0 + st * stage_bytes + 4u * (uint32_t)(pl * a.geo.Q + row0 * P + 4 * c);
 #pragma unroll 4
                 for (int row = row0; row < rows; row += 2) {
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
@@ -333,7 +334,9 @@ template <int P> __global__ void __launch_bounds__(kEsThreads, 1) erode_stream_k
     }
     __syncthreads();
     if (warp >= kEsWarps) {
-        EsProducer<P> io{a, s_ob, s_words, s_live, s_list, s_off, full, empty, &s_stop, ring0, stage_bytes, axis, X0, U0, W0};
+        const long row = a.gpx, plane = (long)a.gpx * a.wy;
+        EsProducer<P> io{a, s_ob, s_words, s_live, s_list, s_off, full, empty, &s_stop, ring0, stage_bytes, X0, U0, W0,
+                         axis ? a.wz : a.wy, axis ? a.wy : a.wz, axis ? plane : row, axis ? row : plane};
         es_produce(io, k1 - k0, NS);
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         return;
